@@ -391,9 +391,11 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * clusters of the membrane-force kernel, each looping over the objects
  * (0, default: one cluster per object; a small grid leaves most SMs to the
  * fluid kernel running beside it).  LBIB_TUNE_MEMBRANE_THREADS: threads per
- * block of the membrane-force kernel (a multiple of 32 in [32, 256],
- * default 192: fewer threads leave more of each SM to the fluid kernel
- * running beside it).  LBIB_TUNE_FLUID_KERNEL (16-bit storage): 0
+ * block of the membrane-force kernel (a multiple of 32 in [32, 256];
+ * reads 192 until set: while neither it nor LBIB_TUNE_MEMBRANE_GROUP is set
+ * and one block takes an object, the step picks 128 to 1024 by the number
+ * and size of the objects and the length of the fluid update beside them;
+ * fewer threads leave more of each SM to the fluid kernel).  LBIB_TUNE_FLUID_KERNEL (16-bit storage): 0
  * (default) and 1 the two-cells-per-thread kernel (where nx is even and
  * there are no obstacles or inlet), 2 the warp-specialised two-cells kernel
  * (a producer warp streams the populations through shared memory with bulk

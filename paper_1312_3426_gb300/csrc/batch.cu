@@ -88,11 +88,12 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     if (i < s.nn_total) node_step<false>(s, i, (int)((t_base[it.x] + step_off) & 1));
 }
 
-__global__ void __launch_bounds__(IB_THREADS, 4)
+template <bool EG>
+__global__ void __launch_bounds__(1024, 1)
     k_batch_membrane(const SimDev *__restrict__ sims, const int2 *__restrict__ items) {
     cg::cluster_group cl = cg::this_cluster();
     const int2 it = items[blockIdx.x / cl.num_blocks()];  // (simulation, object)
-    membrane_object(sims[it.x], it.y, batch_smem, ClusterTeam());
+    membrane_object<EG>(sims[it.x], it.y, batch_smem, ClusterTeam());
 }
 
 // Several (simulation, object) items per block: group g of block b takes
@@ -105,7 +106,7 @@ __global__ void __launch_bounds__(1024, 1)
     if (k >= n_items) return;  // whole groups only
     const int2 it = items[k];
     const GroupTeam tm{(int)threadIdx.x - g * T, T, g + 1};
-    membrane_object(sims[it.x], it.y, batch_smem + (size_t)g * group_floats, tm);
+    membrane_object<false>(sims[it.x], it.y, batch_smem + (size_t)g * group_floats, tm);
 }
 
 __global__ void k_batch_advance(long long *t_base, int n, int steps) {
@@ -127,11 +128,11 @@ struct BatchPlan {
     int2 *d_items = nullptr;  // fluid (by storage type x obstacles), then node, then membrane items
     int n_flp[8] = {};  // fluid items per kernel variant (see fluid_group)
     int n_fl = 0, n_nd = 0, n_mb = 0;
-    int max_nodes = 0;
+    int max_nodes = 0, max_edges = 0;
     // size classes of the membrane items (largest first): the n_big items
     // within a factor 2 of the largest, and the rest, whose largest has
-    // rest_nodes nodes (0: one class)
-    int n_big = 0, rest_nodes = 0;
+    // rest_nodes nodes and rest_edges edges (0: one class)
+    int n_big = 0, rest_nodes = 0, rest_edges = 0;
     int pf_cell = 0, pf_pair = 0;  // L2 prefetch distances of the fluid launches (work items)
     cudaStream_t aux = nullptr;   // membrane kernel
     cudaStream_t aux2 = nullptr;  // membrane kernel of the smaller size class
@@ -186,11 +187,6 @@ static bool plan_matches(lbib_sim *const *sims, int n, int cluster) {
     return true;
 }
 
-static cudaError_t set_membrane_attrs(size_t smem) {
-    static SmemAttr attr;
-    return attr.ensure((const void *)k_batch_membrane, smem, true);
-}
-
 static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStream_t st) {
     g_plan.release();
     const int nthreads = sims[0]->node_threads;  // node chunk of the batch
@@ -207,7 +203,7 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
         if (e != cudaSuccess) return e;
     }
     std::vector<int2> flp[8], fl, nd, mb;
-    int max_nodes = 0;
+    int max_nodes = 0, max_edges = 0;
     for (int i = 0; i < n; ++i) {
         const lbib_sim *s = sims[i];
         const int grp = fluid_group(s);
@@ -218,6 +214,7 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
             for (int f = 0; f < s->nn_total; f += nthreads) nd.push_back(make_int2(i, f));
             for (int o = 0; o < (int)s->objs.size(); ++o) mb.push_back(make_int2(i, o));
             max_nodes = std::max(max_nodes, s->max_nodes);
+            max_edges = std::max(max_edges, s->max_edges);
         }
     }
     // largest objects first: their clusters start in the first wave and the
@@ -262,11 +259,15 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
         g_plan.pf_pair = sms;          // 1 block per SM ahead (3 resident)
     }
     g_plan.max_nodes = max_nodes;
-    g_plan.n_big = 0;
-    while (g_plan.n_big < (int)mb.size() && 2 * sims[mb[g_plan.n_big].x]->objs[mb[g_plan.n_big].y].nn > max_nodes)
-        ++g_plan.n_big;
-    g_plan.rest_nodes = g_plan.n_big < (int)mb.size() ? sims[mb[g_plan.n_big].x]->objs[mb[g_plan.n_big].y].nn : 0;
-    return g_plan.n_mb ? set_membrane_attrs(ib_smem_bytes(max_nodes)) : cudaSuccess;
+    g_plan.max_edges = max_edges;
+    auto nodes_of = [&](const int2 &it) { return sims[it.x]->objs[it.y].nn; };
+    g_plan.n_big = g_plan.rest_nodes = g_plan.rest_edges = 0;
+    while (g_plan.n_big < (int)mb.size() && 2 * nodes_of(mb[g_plan.n_big]) > max_nodes) ++g_plan.n_big;
+    for (size_t k = g_plan.n_big; k < mb.size(); ++k) {
+        g_plan.rest_nodes = std::max(g_plan.rest_nodes, nodes_of(mb[k]));
+        g_plan.rest_edges = std::max(g_plan.rest_edges, sims[mb[k].x]->topo[sims[mb[k].x]->objs[mb[k].y].tid].ne);
+    }
+    return cudaSuccess;
 }
 
 static cudaError_t launch_repulsion_batch(cudaStream_t st) {
@@ -279,10 +280,9 @@ static cudaError_t launch_repulsion_batch(cudaStream_t st) {
 }
 
 // Membrane items [first, first + n) with up to G per block, each with a
-// shared-memory slice for max_nodes nodes (G drops to what fits).
-static cudaError_t launch_membrane_groups(cudaStream_t st, int first, int n, int max_nodes, int G) {
-    const size_t per = ib_smem_bytes(max_nodes);
-    while (G > 1 && (G * g_plan.mthreads > 1024 || per * G > (size_t)227 * 1024)) --G;
+// shared-memory slice of `per` bytes (G drops to what fits).
+static cudaError_t launch_membrane_groups(cudaStream_t st, int first, int n, size_t per, int G) {
+    while (G > 1 && (G * g_plan.mthreads > 1024 || per * G > IB_SMEM_MAX)) --G;
     static SmemAttr gattr;
     cudaError_t e = gattr.ensure((const void *)k_batch_membrane_groups, per * G, false);
     if (e != cudaSuccess) return e;
@@ -301,26 +301,32 @@ static cudaError_t launch_membrane_groups(cudaStream_t st, int first, int n, int
 static cudaError_t launch_membrane_batch(cudaStream_t st) {
     if (g_plan.n_mb == 0) return cudaSuccess;
     const int G = g_plan.mgroup;
-    const size_t per = ib_smem_bytes(g_plan.max_nodes);
-    if (G > 1 && g_plan.n_big < g_plan.n_mb) {
+    const size_t per = ib_smem_bytes(g_plan.max_nodes, g_plan.max_edges);
+    if (G > 1 && g_plan.n_big < g_plan.n_mb && per <= IB_SMEM_MAX) {
         cudaError_t e;
         if ((e = cudaStreamWaitEvent(g_plan.aux2, g_plan.ev_nodes, 0)) != cudaSuccess) return e;
-        if ((e = launch_membrane_groups(g_plan.aux2, g_plan.n_big, g_plan.n_mb - g_plan.n_big, g_plan.rest_nodes, G)) !=
-            cudaSuccess)
+        if ((e = launch_membrane_groups(g_plan.aux2, g_plan.n_big, g_plan.n_mb - g_plan.n_big,
+                                        ib_smem_bytes(g_plan.rest_nodes, g_plan.rest_edges), G)) != cudaSuccess)
             return e;
         if ((e = cudaEventRecord(g_plan.ev_rest, g_plan.aux2)) != cudaSuccess) return e;
-        if ((e = launch_membrane_groups(st, 0, g_plan.n_big, g_plan.max_nodes, G)) != cudaSuccess) return e;
+        if ((e = launch_membrane_groups(st, 0, g_plan.n_big, per, G)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(st, g_plan.ev_rest, 0)) != cudaSuccess) return e;
         return launch_repulsion_batch(st);
     }
-    if (G > 1 && G * g_plan.mthreads <= 1024 && per * G <= (size_t)227 * 1024) {
-        cudaError_t e = launch_membrane_groups(st, 0, g_plan.n_mb, g_plan.max_nodes, G);
+    if (G > 1 && G * g_plan.mthreads <= 1024 && per * G <= IB_SMEM_MAX) {
+        cudaError_t e = launch_membrane_groups(st, 0, g_plan.n_mb, per, G);
         return e == cudaSuccess ? launch_repulsion_batch(st) : e;
     }
+    const bool global = membrane_in_global(g_plan.max_nodes, g_plan.max_edges, g_plan.cluster);
+    const size_t smem = global ? ib_smem_bytes(g_plan.max_nodes, 0) : per;
+    static SmemAttr attr[2];
+    cudaError_t e = attr[global].ensure(
+        global ? (const void *)k_batch_membrane<true> : (const void *)k_batch_membrane<false>, smem, true);
+    if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)(g_plan.n_mb * g_plan.cluster));
     cfg.blockDim = dim3((unsigned)g_plan.mthreads);
-    cfg.dynamicSmemBytes = ib_smem_bytes(g_plan.max_nodes);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cudaLaunchAttribute at[1];
     at[0].id = cudaLaunchAttributeClusterDimension;
@@ -329,8 +335,8 @@ static cudaError_t launch_membrane_batch(cudaStream_t st) {
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    cudaError_t e = cudaLaunchKernelEx(&cfg, k_batch_membrane, (const SimDev *)g_plan.d_sims,
-                                       (const int2 *)(g_plan.d_items + g_plan.n_fl + g_plan.n_nd));
+    e = cudaLaunchKernelEx(&cfg, global ? k_batch_membrane<true> : k_batch_membrane<false>,
+                           (const SimDev *)g_plan.d_sims, (const int2 *)(g_plan.d_items + g_plan.n_fl + g_plan.n_nd));
     // object-object repulsion of the simulations that set it (per simulation)
     return e == cudaSuccess ? launch_repulsion_batch(st) : e;
 }
@@ -434,6 +440,17 @@ extern "C" lbib_status lbib_batch_step(lbib_sim *const *sims, int n, int n_steps
     }
     cudaError_t e = cudaSuccess;
     const int cluster = sims[0]->cluster;
+    int max_nodes = 0, max_edges = 0;
+    for (int i = 0; i < n; ++i)
+        if (!sims[i]->objs.empty()) {
+            max_nodes = std::max(max_nodes, sims[i]->max_nodes);
+            max_edges = std::max(max_edges, sims[i]->max_edges);
+        }
+    if (membrane_in_global(max_nodes, max_edges, cluster))
+        for (int i = 0; i < n; ++i) {
+            const lbib_status r = sims[i]->objs.empty() ? LBIB_OK : sim_edge_scratch(sims[i]);
+            if (r != LBIB_OK) return r;
+        }
     if (!plan_matches(sims, n, cluster)) e = build_plan(sims, n, cluster, st);
     if (g_plan.mthreads != sims[0]->membrane_threads || g_plan.mgroup != sims[0]->membrane_group) {
         g_plan.mthreads = sims[0]->membrane_threads;  // captured in the graph

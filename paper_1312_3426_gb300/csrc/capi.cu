@@ -51,10 +51,16 @@ bool fluid_layout(const lbib_fluid_params &p, FluidLayout &L) {
     return true;
 }
 
-// device records of a template: triangles (int4), and per edge its hinge
-// nodes (int4) and constants (float4)
+size_t edge_stride(const Topology &T) { return align_up((size_t)T.ne, 32); }
+
+// a mesh whose edge or triangle numbers do not fit in 16 bits
+bool wide_ring(const Topology &T) { return T.ne > 65536 || T.nt > 65536; }
+
+// device records of a template: triangles (int4), the three edge arrays, the
+// node slots (int4) and the walks (8 or 16 bytes a record)
 size_t template_bytes(const Topology &T) {
-    return align_up((size_t)T.nt * 16, 256) + 2 * align_up((size_t)T.ne * 16, 256);
+    return align_up((size_t)T.nt * 16, 256) + align_up(edge_stride(T) * 40, 256) +
+           align_up(T.slots.size() / 3 * 16, 256) + align_up(T.rings.size() * (wide_ring(T) ? 4 : 2), 256);
 }
 
 lbib_status fail(lbib_sim *s, lbib_status code, const std::string &msg) {
@@ -156,25 +162,33 @@ lbib_status sim_upload(lbib_sim *s) {
         const int nobj = (int)s->objs.size();
         if (nobj > s->d_obj_cap) {
             const int cap = std::max(nobj, 2 * s->d_obj_cap);
-            cudaFree(s->d_obj);
-            cudaFree(s->d_fext);
-            cudaFree(s->d_analyze);
-            s->d_obj = nullptr;
-            s->d_fext = nullptr;
-            s->d_analyze = nullptr;
+            cudaFree(s->d_mem);
+            s->d_mem = nullptr;
             s->d_obj_cap = 0;
-            LBIB_CUDA(s, cudaMalloc(&s->d_obj, cap * sizeof(ObjDev)), "object table");
-            LBIB_CUDA(s, cudaMalloc(&s->d_fext, cap * 3 * sizeof(float)), "object forces");
-            LBIB_CUDA(s, cudaMalloc(&s->d_analyze, cap * 14 * sizeof(double)), "analysis buffer");
+            // one allocation: membrane records, read-out buffer, object table, forces
+            LBIB_CUDA(s, cudaMalloc(&s->d_mem, cap * (sizeof(MemDev) + 14 * sizeof(double) + sizeof(ObjDev) +
+                                                      3 * sizeof(float))), "object tables");
+            s->d_analyze = (double *)(s->d_mem + cap);
+            s->d_obj = (ObjDev *)(s->d_analyze + 14 * (size_t)cap);
+            s->d_fext = (float *)(s->d_obj + cap);
             s->d_obj_cap = cap;
             s->fext_dirty = true;
         }
+        std::vector<MemDev> mem(nobj);
+        for (int o = 0; o < nobj; ++o) {
+            mem[o] = s->tpl_mem_dev[s->objs[o].tid];
+            mem[o].first = s->objs[o].first;
+        }
+        if (nobj > 0)
+            LBIB_CUDA(s, cudaMemcpyAsync(s->d_mem, mem.data(), nobj * sizeof(MemDev), cudaMemcpyHostToDevice, s->stream),
+                      "membrane table");
         if (nobj > 0)
             LBIB_CUDA(s, cudaMemcpyAsync(s->d_obj, s->objs.data(), nobj * sizeof(ObjDev), cudaMemcpyHostToDevice,
                                          s->stream), "object table");
         LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "tables");
         s->d.tpl = s->d_tpl;
         s->d.obj = s->d_obj;
+        s->d.mem = s->d_mem;
         s->d.fext = s->d_fext;
         s->d.nobj = nobj;
         // repulsion buffers: boxes [nobj][8], a pair list of 32 per object
@@ -270,10 +284,29 @@ lbib_status sim_upload(lbib_sim *s) {
     return LBIB_OK;
 }
 
+// Global memory for the edge scalars of every object, for launches that do
+// not keep them in shared memory (membrane_in_global).
+lbib_status sim_edge_scratch(lbib_sim *s) {
+    const size_t stride = align_up(membrane_scalar_bytes(s->max_edges), 16), bytes = s->objs.size() * stride;
+    if (bytes > s->edge_bytes) {
+        if (s->d.edge_scal) cudaFree(s->d.edge_scal);
+        s->d.edge_scal = nullptr;
+        s->edge_bytes = 0;
+        LBIB_CUDA(s, cudaMalloc(&s->d.edge_scal, bytes), "edge scalars");
+        s->edge_bytes = bytes;
+    }
+    s->d.edge_stride = stride;
+    return LBIB_OK;
+}
+
 lbib_status sim_prepare_step(lbib_sim *s) {
     if (!s->fluid_ready) return fail(s, LBIB_ERR_STATE, "lbib_fluid_init must precede lbib_step");
     lbib_status r = sim_upload(s);
     if (r != LBIB_OK) return r;
+    if (!s->objs.empty() && membrane_in_global(s->max_nodes, s->max_edges, s->cluster)) {
+        r = sim_edge_scratch(s);
+        if (r != LBIB_OK) return r;
+    }
     if (s->ufield_stale) {
         LBIB_CUDA(s, launch_fields(s->d, (int)(s->t & 1), s->gmode, nullptr, nullptr, 1, s->stream), "velocity samples");
         s->ufield_stale = false;
@@ -430,14 +463,13 @@ void lbib_destroy(lbib_sim *s) {
     }
     for (auto &t : s->tpl_mem) cudaFree(t);
     if (s->d_tpl) cudaFree(s->d_tpl);
-    if (s->d_obj) cudaFree(s->d_obj);
-    if (s->d_fext) cudaFree(s->d_fext);
-    if (s->d_analyze) cudaFree(s->d_analyze);
+    if (s->d_mem) cudaFree(s->d_mem);
 
     for (cudaEvent_t e : s->prof_ev) cudaEventDestroy(e);
     for (cudaEvent_t e : s->prof_aux) cudaEventDestroy(e);
     if (s->dnodes) cudaFree(s->dnodes);
     if (s->rep_mem) cudaFree(s->rep_mem);
+    if (s->d.edge_scal) cudaFree(s->d.edge_scal);
     if (s->solid_mem) cudaFree(s->solid_mem);
     if (s->fluid_mem) cudaFree(s->fluid_mem);
     delete s;
@@ -455,6 +487,7 @@ lbib_status lbib_template_create(lbib_sim *s, int tid, const double *xyz, int nn
     Topology T;
     std::string err;
     if (!build_template(xyz, nn, tris, nt, stretch, T, err)) return fail(s, LBIB_ERR_MESH, err);
+    ring_walks(T, RING_START);
     // device records, one allocation
     const size_t bytes = template_bytes(T);
     void *mem = nullptr;
@@ -474,8 +507,10 @@ lbib_status lbib_template_create(lbib_sim *s, int tid, const double *xyz, int nn
         std::memcpy(&i, &f, 4);
         return i;
     };
-    std::vector<int32_t> tri4(4 * (size_t)nt), quad4(4 * (size_t)T.ne);
-    std::vector<float> hinge4(4 * (size_t)T.ne);
+    std::vector<int32_t> tri4(4 * (size_t)nt);
+    const size_t es = edge_stride(T);
+    std::vector<int32_t> edge(10 * es, 0);  // quads (4 es), rest state (4 es), rest areas of the owned triangles (2 es)
+    std::vector<char> owned(nt, 0);
     // device records in the conflict-free evaluation order of each kind
     for (int j = 0; j < nt; ++j) {
         const int t = T.tri_order[j];
@@ -486,15 +521,34 @@ lbib_status lbib_template_create(lbib_sim *s, int tid, const double *xyz, int nn
     // carries both (the stretching and the bending of that edge)
     for (int j = 0; j < T.ne; ++j) {
         const int e = T.quad_order[j];
-        for (int k = 0; k < 4; ++k) quad4[4 * j + k] = T.quads[4 * e + k];
-        hinge4[4 * j] = (float)T.L0[e];
-        hinge4[4 * j + 1] = (float)(1.0 / T.L0[e]);
-        hinge4[4 * j + 2] = (float)(1.0 / T.theta0[e]);
-        hinge4[4 * j + 3] = 0.f;
+        const int *q = &T.quads[4 * e];
+        int32_t *r = &edge[4 * (size_t)j], *h = &edge[4 * (es + j)], *s0 = &edge[8 * es + 2 * j];
+        r[0] = q[0] | q[1] << 16;
+        r[1] = q[2] | q[3] << 16;
+        for (int k = 0; k < 2; ++k) {  // the first edge of a triangle in this order owns it
+            const int t = T.quad_tris[2 * e + k];
+            r[2 + k] = owned[t] ? -1 : t;
+            s0[k] = fbits(T.S0[t]);
+            owned[t] = 1;
+        }
+        h[0] = fbits(T.L0[e]);
+        h[1] = fbits(1.0 / T.L0[e]);
+        h[2] = fbits(1.0 / T.theta0[e]);
+        h[3] = fbits(3.14159265358979323846 - T.theta0[e]);
     }
+    const size_t n_slots = T.slots.size() / 3;
+    std::vector<int32_t> slot4(4 * n_slots);
+    for (size_t j = 0; j < n_slots; ++j)
+        for (int k = 0; k < 3; ++k) slot4[4 * j + k] = T.slots[3 * j + k];
+    std::vector<uint32_t> ring;
+    if (wide_ring(T)) ring = T.rings;
+    else
+        for (size_t j = 0; j < T.rings.size(); j += 4)
+            ring.insert(ring.end(), {T.rings[j] | T.rings[j + 1] << 16, T.rings[j + 2] | T.rings[j + 3] << 16});
     const size_t o_tri = put(tri4.data(), tri4.size() * 4);
-    const size_t o_quad = put(quad4.data(), quad4.size() * 4);
-    const size_t o_hinge = put(hinge4.data(), hinge4.size() * 4);
+    const size_t o_edge = put(edge.data(), edge.size() * 4);
+    const size_t o_slot = put(slot4.data(), slot4.size() * 4);
+    const size_t o_ring = put(ring.data(), ring.size() * 4);
     cudaError_t e = cudaMemcpyAsync(mem, host.data(), bytes, cudaMemcpyHostToDevice, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) {
@@ -504,24 +558,31 @@ lbib_status lbib_template_create(lbib_sim *s, int tid, const double *xyz, int nn
     char *b = (char *)mem;
     dv.nn = T.nn;
     dv.nt = T.nt;
-    dv.ks = (float)ks;
-    dv.kb = (float)kb;
-    dv.kal = (float)kal;
-    dv.kag = (float)kag;
-    dv.kv = (float)kv;
-    dv.nonlinear = nonlinear ? 1 : 0;
-    dv.kal_altitude = 0;
-    dv.Sg0 = T.Sg0;
-    dv.V0 = T.V0;
-    dv.ne = T.ne;
     dv.tri = (const int4 *)(b + o_tri);
-    dv.quad = (const int4 *)(b + o_quad);
-    dv.hinge = (const float4 *)(b + o_hinge);
+    MemDev md{};  // first is set per object
+    md.nn = T.nn;
+    md.ne = T.ne;
+    md.n_slots = (int)n_slots;
+    md.edge = (const int4 *)(b + o_edge);
+    md.ring = b + o_ring;
+    md.slot = (const int4 *)(b + o_slot);
+    md.edge_stride = (int)es;
+    md.flags = (nonlinear ? MEM_NONLINEAR : 0) | (wide_ring(T) ? MEM_WIDE : 0);
+    md.ks = (float)ks;
+    md.kb = (float)kb;
+    md.kal = (float)kal;
+    md.kag = (float)kag;
+    md.kv = (float)kv;
+    md.Sg0 = T.Sg0;
+    md.V0 = T.V0;
+    s->tpl_mem_dev.push_back(md);
+    const int ne = T.ne;
     s->topo.push_back(std::move(T));
     s->tpl_dev.push_back(dv);
     s->tpl_mem.push_back(mem);
     s->tpl_bytes += bytes;
     s->max_nodes = std::max(s->max_nodes, nn);
+    s->max_edges = std::max(s->max_edges, ne);
     s->tables_dirty = true;
     return LBIB_OK;
 }
@@ -619,7 +680,8 @@ lbib_status lbib_object_add(lbib_sim *s, int oid, int tid, const double origin[3
 lbib_status lbib_template_set_kal_direction(lbib_sim *s, int tid, int altitude) {
     LBIB_GUARD(s);
     if (tid < 0 || tid >= (int)s->tpl_dev.size()) return fail(s, LBIB_ERR_ID, "unknown template id");
-    s->tpl_dev[tid].kal_altitude = altitude ? 1 : 0;
+    int &flags = s->tpl_mem_dev[tid].flags;
+    flags = altitude ? flags | MEM_ALTITUDE : flags & ~MEM_ALTITUDE;
     s->tables_dirty = true;
     s->fel_valid = false;
     return LBIB_OK;
@@ -768,7 +830,11 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
         if (r != LBIB_OK) return r;
         LBIB_CUDA(s, cudaEventRecord(ev[0], st), "profile event");
     }
-    LBIB_CUDA(s, launch_membrane(s->d, s->max_nodes, s->cluster, s->membrane_clusters, s->membrane_threads,
+    const int threads = s->membrane_auto && s->cluster == 1
+                            ? membrane_threads((int)s->objs.size(), s->max_edges,
+                                               s->overlap ? fluid_time_us(s->d.nf, s->p.precision) : 0.0)
+                            : s->membrane_threads;
+    LBIB_CUDA(s, launch_membrane(s->d, s->max_nodes, s->max_edges, s->cluster, s->membrane_clusters, threads,
                                  s->membrane_group, st), "membrane forces");
     LBIB_CUDA(s, launch_repulsion(s->d, s->max_nodes, st), "repulsion");
     if (ev) LBIB_CUDA(s, cudaEventRecord(ev[1], st), "profile event");
@@ -1075,7 +1141,7 @@ lbib_status lbib_info(const lbib_sim *s, int64_t out[8]) {
     out[2] = s->nn_total;
     out[3] = s->d.nf;
     out[4] = s->t;
-    out[5] = (int64_t)(s->fluid_bytes + s->tpl_bytes + s->node_bytes + s->rep_bytes +
+    out[5] = (int64_t)(s->fluid_bytes + s->tpl_bytes + s->node_bytes + s->rep_bytes + s->edge_bytes +
                        (s->solid_mem ? (size_t)s->d.nwords * 4 : 0));
     out[6] = s->p.precision;
     out[7] = fluid_kernel_kind(s->d);
@@ -1185,6 +1251,7 @@ lbib_status lbib_set_tuning(lbib_sim *s, int key, int value) {
     if (key == LBIB_TUNE_MEMBRANE_THREADS) {
         if (value < 32 || value > IB_THREADS || value % 32) return fail(s, LBIB_ERR_ARG, "membrane threads must be a multiple of 32 in [32, 256]");
         s->membrane_threads = value;
+        s->membrane_auto = false;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_MEMBRANE_CLUSTERS) {
@@ -1200,6 +1267,7 @@ lbib_status lbib_set_tuning(lbib_sim *s, int key, int value) {
     if (key == LBIB_TUNE_MEMBRANE_GROUP) {
         if (value < 1 || value > 15) return fail(s, LBIB_ERR_ARG, "membrane group must be in [1, 15]");
         s->membrane_group = value;
+        s->membrane_auto = false;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_NODE_THREADS) {

@@ -54,8 +54,7 @@ int fluid_kernel_kind(const SimDev &s) {
     return 1;
 }
 
-// SM count of the current device (cached per device).
-static int device_sms() {
+int device_sms() {
     static std::mutex mu;
     static int sms[64] = {};
     int dev = 0;

@@ -9,11 +9,12 @@ extern __shared__ float ib_smem[];
 
 // Cluster c takes objects c, c + n_clusters, ... (a grid smaller than the
 // object count leaves SMs to the fluid kernel that runs beside it).
-__global__ void __launch_bounds__(IB_THREADS, 4) k_membrane(SimDev s) {
+template <bool EG>
+__global__ void __launch_bounds__(1024, 1) k_membrane(SimDev s) {
     const ClusterTeam tm;
     const int C = tm.ranks();
     const int n_clusters = (int)(gridDim.x / C);
-    for (int o = (int)(blockIdx.x / C); o < s.nobj; o += n_clusters) membrane_object(s, o, ib_smem, tm);
+    for (int o = (int)(blockIdx.x / C); o < s.nobj; o += n_clusters) membrane_object<EG>(s, o, ib_smem, tm);
 }
 
 // Several objects per block: group g (threads [g T, (g + 1) T)) of block b
@@ -25,7 +26,7 @@ __global__ void __launch_bounds__(1024, 1) k_membrane_groups(SimDev s, int T, in
     const int o = (int)blockIdx.x * G + g;
     if (o >= s.nobj) return;  // whole groups only: no barrier is shared with another group
     const GroupTeam tm{(int)threadIdx.x - g * T, T, g + 1};
-    membrane_object(s, o, ib_smem + (size_t)g * group_floats, tm);
+    membrane_object<false>(s, o, ib_smem + (size_t)g * group_floats, tm);
 }
 
 // NT nodes per block (LBIB_TUNE_NODE_THREADS: 32, 64, 128 or 256); EARLY:
@@ -36,12 +37,43 @@ __global__ void __launch_bounds__(NT, 1024 / NT) k_nodes(SimDev s, int par) {
     if (i < s.nn_total) node_step<EARLY>(s, i, par);
 }
 
-cudaError_t launch_membrane(const SimDev &s, int max_nodes, int cluster, int max_clusters, int threads, int group,
-                            cudaStream_t st) {
+bool membrane_in_global(int max_nodes, int max_edges, int cluster) {
+    return cluster > 1 || ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX;
+}
+
+size_t membrane_scalar_bytes(int max_edges) { return ib_scalar_bytes(max_edges); }
+
+// The membrane kernel takes about 10 us plus 3.5 us for every round of the
+// block over the edges (beside the fluid kernel; a level-3 cell of 1920
+// edges: 66 us at 128 threads, 47 at 256, 24 at 1024).  It is hidden while
+// it is shorter than the fluid update, and every thread it holds is one the
+// fluid blocks lack: so the fewest threads that keep it hidden, and at least
+// 128 (192 where the objects come in many waves).  Where none does, the
+// step waits for it: as many as help (two edges a thread), while all objects
+// together take no more than 256 threads per SM.  Steps, this rule against
+// 192 threads for all: 64x48x48 with 3 cells (FP16) 20.8 against 31.2 us,
+// 160x96x96 with 20 cells (FP32) 47.7 against 56.4, 256x128x128 with 60
+// level-4 cells (FP32) 120.9 against 147.6, 200 level-3 cells 124.4 against
+// 125.9.
+int membrane_threads(int nobj, int max_edges, double fluid_us) {
+    static const int choice[] = {128, 192, 256, 384, 512, 768, 1024};
+    const int sms = device_sms();
+    int best = nobj > 2 * sms ? 192 : 128;
+    for (int t : choice) {
+        if (t <= best) continue;
+        const int rounds = (max_edges + best - 1) / best;
+        if (10.0 + 3.5 * rounds <= fluid_us || 2 * best >= max_edges || (int64_t)t * nobj > (int64_t)256 * sms) break;
+        best = t;
+    }
+    return best;
+}
+
+cudaError_t launch_membrane(const SimDev &s, int max_nodes, int max_edges, int cluster, int max_clusters, int threads,
+                            int group, cudaStream_t st) {
     if (s.nobj == 0) return cudaSuccess;
     // as many objects per block as fit (threads and shared memory), at most `group`
-    const size_t per = ib_smem_bytes(max_nodes);  // a multiple of 16 bytes
-    while (group > 1 && (group * threads > 1024 || group > 15 || per * (size_t)group > 227 * 1024)) --group;
+    const size_t per = ib_smem_bytes(max_nodes, max_edges);  // a multiple of 16 bytes
+    while (group > 1 && (group * threads > 1024 || group > 15 || per * (size_t)group > IB_SMEM_MAX)) --group;
     if (group > 1) {  // several objects per block (cluster size and cluster count do not apply)
         const size_t smem = per * (size_t)group;
         static SmemAttr gattr;
@@ -51,9 +83,11 @@ cudaError_t launch_membrane(const SimDev &s, int max_nodes, int cluster, int max
         k_membrane_groups<<<blocks, group * threads, smem, st>>>(s, threads, (int)(per / sizeof(float)));
         return cudaGetLastError();
     }
-    const size_t smem = per;
-    static SmemAttr attr;
-    cudaError_t ea = attr.ensure((const void *)k_membrane, smem, true);
+    const bool global = membrane_in_global(max_nodes, max_edges, cluster);
+    const size_t smem = global ? ib_smem_bytes(max_nodes, 0) : per;
+    static SmemAttr attr[2];
+    cudaError_t ea = attr[global].ensure(global ? (const void *)k_membrane<true> : (const void *)k_membrane<false>, smem,
+                                         true);
     if (ea != cudaSuccess) return ea;
     cudaLaunchConfig_t cfg = {};
     const int n_clusters = (max_clusters > 0 && max_clusters < s.nobj) ? max_clusters : s.nobj;
@@ -68,7 +102,7 @@ cudaError_t launch_membrane(const SimDev &s, int max_nodes, int cluster, int max
     at[0].val.clusterDim.z = 1;
     cfg.attrs = at;
     cfg.numAttrs = 1;
-    return cudaLaunchKernelEx(&cfg, k_membrane, s);
+    return cudaLaunchKernelEx(&cfg, global ? k_membrane<true> : k_membrane<false>, s);
 }
 
 cudaError_t launch_nodes(const SimDev &s, int par, int threads, cudaStream_t st, bool pdl) {

@@ -40,7 +40,7 @@ namespace lbib {
 
 constexpr int NQ = 19;
 constexpr int FLUID_THREADS = 256;
-constexpr int IB_THREADS = 256;          // largest block of the object kernels
+constexpr int IB_THREADS = 256;          // largest LBIB_TUNE_MEMBRANE_THREADS
 constexpr int IB_THREADS_DEFAULT = 256;  // node kernel block (LBIB_TUNE_NODE_THREADS)
 constexpr int MAX_TEMPLATE_NODES = 5120;  // 11 floats of shared memory per node
 constexpr int ACTIVE_RESET_STEPS = 128;    // period of the active-cell re-marking
@@ -71,22 +71,45 @@ enum : uint32_t {
     ST_PAIRS = 8u,        // more close object pairs than the repulsion pair list holds
 };
 
-// Element lists of one template (device), all node ids local to an object,
-// each in the bank-aware evaluation order of topology.cpp:
-//   tri:        (a, b, c, rest area S0 as float bits), inward-ordered as given
-//   quad:       per edge (b, c), b < c: (a, b, c, d), where (a,b,c) and
-//               (d,c,b) are the inward cyclic orders of the two triangles
-//               sharing it
-//   hinge:      per edge, (rest length L0, 1/L0, 1/rest inner angle, 0)
+// Element lists of one template (device), all node ids local to an object:
+//   tri:        (a, b, c, rest area S0 as float bits), inward-ordered, in the
+//               bank-aware evaluation order of topology.cpp (read-outs)
 struct TplDev {
-    int nn, nt, ne;
-    float ks, kb, kal, kag, kv;
-    int nonlinear;
-    int kal_altitude;  // local-area force along the altitudes (else centroid -> vertex)
-    double Sg0, V0;
+    int nn, nt;
     const int4 *tri;
-    const int4 *quad;
-    const float4 *hinge;
+};
+
+// Everything the membrane kernel needs of one object, in one record (one
+// load instead of object, then template): its nodes, its template's element
+// lists (node ids local to the object) and moduli.
+//   edge:       per edge (b, c), b < c, in the bank-aware order, three arrays of
+//               16-byte vectors, edge_stride apart: (a | b << 16, c | d << 16, t1, t2),
+//               where (a,b,c) and (d,c,b) are the inward cyclic orders of the
+//               two triangles sharing it, t1 and t2 their numbers where this
+//               edge owns them (each triangle is owned by one edge), else -1;
+//               (rest length L0, 1/L0, 1/theta0, pi - theta0), theta0 the rest
+//               inner angle; the rest areas of t1 and t2 (8-byte vectors)
+//   slot:       per slot of the node pass (nodes by number of records, so the
+//               lanes of a warp walk equally far; padded to whole warps):
+//               (node or -1, its first record, number of records, 0)
+//   ring:       the records of the walk around each node v: the next neighbour
+//               q (with the RING_START flag), edge (v,q), edge (p,q) opposite v,
+//               triangle (v,p,q), p the neighbour before; record j of the 32
+//               slots of a warp lie side by side (stride 32).  16 bits each
+//               (uint2), or 32 bits (uint4, MEM_WIDE) where a mesh has more
+//               than 65536 edges or triangles.  Edges count in the order of
+//               `edge`.
+constexpr uint32_t RING_START = 0x8000u;  // a fan starts at q: no triangle
+enum : int { MEM_NONLINEAR = 1, MEM_ALTITUDE = 2, MEM_WIDE = 4 };
+struct alignas(16) MemDev {
+    int first, nn, ne, n_slots;
+    const int4 *edge;
+    const void *ring;
+    const int4 *slot;
+    int edge_stride, flags;  // MEM_ALTITUDE: local-area force along the altitudes (else centroid -> vertex)
+    float ks, kb, kal, kag;
+    double Sg0, V0;
+    float kv, pad[3];
 };
 
 // One object: its template, first global node, node count and 1/m.
@@ -134,11 +157,14 @@ struct SimDev {
     float4 *ufield;
     float *Xh, *Xl, *Vh, *Vl; // [3][nn_total] each
     float *Fel;               // [3][nn_total] membrane force of the current step
+    char *edge_scal;          // [nobj][edge_stride] edge and triangle scalars, where shared memory does not serve
+    size_t edge_stride;       // bytes
     const int *node_obj;      // [nn_total] object of each node
     int nn_total, nobj;
     const ObjDev *obj;
     const float *fext;        // [nobj][3] external force per node of each object
     const TplDev *tpl;
+    const MemDev *mem;        // [nobj]
     uint32_t *status;
     double *dropped;          // [3]
     // soft-sphere repulsion (a, n, cutoff): object-object and object-wall
@@ -249,12 +275,24 @@ cudaError_t launch_mass_partials(const SimDev &s, int pop_par, double *part, int
 
 // ---- launchers (ib.cu) -----------------------------------------------------
 // membrane part: clusters of `cluster` blocks, one per object or at most
-// max_clusters (> 0) looping over the objects (max_nodes sizes shared
-// memory); coupling part: one thread per node
-// threads: block size (a multiple of 32, at most IB_THREADS)
+// max_clusters (> 0) looping over the objects (max_nodes and max_edges size
+// shared memory); coupling part: one thread per node
+// threads: block size (a multiple of 32, at most 1024)
 // group > 1: `group` objects per block of group * threads threads instead
-cudaError_t launch_membrane(const SimDev &s, int max_nodes, int cluster, int max_clusters, int threads, int group,
-                            cudaStream_t st);
+cudaError_t launch_membrane(const SimDev &s, int max_nodes, int max_edges, int cluster, int max_clusters, int threads,
+                            int group, cudaStream_t st);
+// whether a launch of one object per cluster keeps the edge scalars in
+// SimDev::edge_scal: several blocks per object, or more than one block's
+// shared memory holds
+bool membrane_in_global(int max_nodes, int max_edges, int cluster);
+size_t membrane_scalar_bytes(int max_edges);  // per object
+// Threads per object of a membrane launch of nobj objects (one per block)
+// beside a fluid update of fluid_us microseconds (0: nothing beside it).
+int membrane_threads(int nobj, int max_edges, double fluid_us);
+// Time of the fluid update of nf cells: its populations in and out at 6 TB/s.
+inline double fluid_time_us(int64_t nf, int prec) { return (double)nf * 38 * (prec == LBIB_POP_F32 ? 4 : 2) / 6.0e6; }
+// SM count of the current device (cached per device)
+int device_sms();
 // pdl: launch with programmatic stream serialization (only right after the
 // previous step's fluid kernel, a mask rebuild or a membrane kernel)
 cudaError_t launch_nodes(const SimDev &s, int par, int threads, cudaStream_t st, bool pdl = false);

@@ -25,9 +25,12 @@ struct lbib_sim {
 
     std::vector<lbib::Topology> topo;   // host copy of every template
     std::vector<lbib::TplDev> tpl_dev;  // device descriptors of the templates
+    std::vector<lbib::MemDev> tpl_mem_dev;  // membrane records of the templates (first: per object)
     std::vector<void *> tpl_mem;        // device records of every template
     size_t tpl_bytes = 0;
     int max_nodes = 0;                  // largest template
+    int max_edges = 0;
+    size_t edge_bytes = 0;              // of SimDev::edge_scal
 
     std::vector<lbib::ObjDev> objs;
     int nn_total = 0;
@@ -38,8 +41,9 @@ struct lbib_sim {
     float *dnodes = nullptr;     // Xh, Xl, Vh, Vl, Fel, each [3][nn_total], then node_obj [nn_total]
     int dev_nn_cap = 0;
     size_t node_bytes = 0;
-    lbib::ObjDev *d_obj = nullptr;
     lbib::TplDev *d_tpl = nullptr;
+    lbib::MemDev *d_mem = nullptr;  // one allocation with d_analyze, d_obj and d_fext
+    lbib::ObjDev *d_obj = nullptr;
     std::vector<float> fext;     // [nobj][3]
     float *fext_pinned = nullptr;      // page-locked staging of fext for asynchronous uploads
     size_t fext_pinned_cap = 0;
@@ -73,7 +77,8 @@ struct lbib_sim {
     cudaStream_t side = nullptr;
     bool overlap = true;                // membrane of step t+1 on `aux` during fluid of step t
     int membrane_clusters = 0;          // clusters of the membrane kernel (0: one per object)
-    int membrane_threads = 192;         // block size of the membrane kernel (per object)
+    int membrane_threads = 192;         // block size of the membrane kernel (per object) ...
+    bool membrane_auto = true;          // ... unless neither it nor the group was set: membrane_threads()
     int membrane_group = 1;             // objects per block of the membrane kernel
     bool early_launch = false;          // programmatic dependent launch of the node and fluid kernels
     int node_threads = lbib::IB_THREADS_DEFAULT;  // nodes per block of the node kernel
@@ -105,5 +110,6 @@ lbib_status sim_check_status(lbib_sim *s);
 lbib_status sim_download_nodes(lbib_sim *s);
 lbib_status sim_upload(lbib_sim *s);
 lbib_status sim_prepare_step(lbib_sim *s);
+lbib_status sim_edge_scratch(lbib_sim *s);
 cudaError_t sim_remark(lbib_sim *s, cudaStream_t st);
 }  // namespace lbib

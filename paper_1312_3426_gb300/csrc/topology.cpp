@@ -82,14 +82,14 @@ bool build_template(const double *xyz, int nn, const int32_t *tris, int nt, cons
     // directed edges (from, to) -> apex, sorted by key
     struct DE {
         uint64_t key;
-        int apex;
+        int apex, tri;
     };
     std::vector<DE> de;
     de.reserve(3 * (size_t)nt);
     for (int t = 0; t < nt; ++t)
         for (int k = 0; k < 3; ++k) {
             const uint32_t i = (uint32_t)T.tri[3 * t + k], j = (uint32_t)T.tri[3 * t + (k + 1) % 3];
-            de.push_back({((uint64_t)i << 32) | j, T.tri[3 * t + (k + 2) % 3]});
+            de.push_back({((uint64_t)i << 32) | j, T.tri[3 * t + (k + 2) % 3], t});
         }
     std::sort(de.begin(), de.end(), [](const DE &p, const DE &q) { return p.key < q.key; });
     for (size_t k = 1; k < de.size(); ++k)
@@ -97,16 +97,17 @@ bool build_template(const double *xyz, int nn, const int32_t *tris, int nt, cons
             err = "directed edge used twice: the mesh is non-manifold or inconsistently ordered";
             return false;
         }
-    auto find = [&](uint64_t key) -> int {
+    auto find = [&](uint64_t key) -> const DE * {
         auto it = std::lower_bound(de.begin(), de.end(), key, [](const DE &p, uint64_t k) { return p.key < k; });
-        return (it != de.end() && it->key == key) ? it->apex : -1;
+        return (it != de.end() && it->key == key) ? &*it : nullptr;
     };
     T.edges.clear();
     T.quads.clear();
+    T.quad_tris.clear();
     for (const DE &e : de) {
         const int b = (int)(e.key >> 32), c = (int)(e.key & 0xffffffffu);
-        const int d = find(((uint64_t)(uint32_t)c << 32) | (uint32_t)b);
-        if (d < 0) {
+        const DE *back = find(((uint64_t)(uint32_t)c << 32) | (uint32_t)b);
+        if (!back) {
             err = "edge " + std::to_string(b) + "-" + std::to_string(c) + " has no opposite triangle (open mesh)";
             return false;
         }
@@ -116,7 +117,9 @@ bool build_template(const double *xyz, int nn, const int32_t *tris, int nt, cons
             T.quads.push_back(e.apex);
             T.quads.push_back(b);
             T.quads.push_back(c);
-            T.quads.push_back(d);
+            T.quads.push_back(back->apex);
+            T.quad_tris.push_back(e.tri);
+            T.quad_tris.push_back(back->tri);
         }
     }
     T.ne = (int)(T.edges.size() / 2);
@@ -162,6 +165,73 @@ bool build_template(const double *xyz, int nn, const int32_t *tris, int nt, cons
     T.quad_order = conflict_free_order(T.quads, 4, 32);
     T.tri_order = conflict_free_order(T.tri, 3, 32);
     return true;
+}
+
+void ring_walks(Topology &T, uint32_t start) {
+    // place of edge (i, j) in the device order
+    std::vector<int> place(T.ne);
+    for (int j = 0; j < T.ne; ++j) place[T.quad_order[j]] = j;
+    std::vector<int> first(T.nn + 1, 0);  // edges are lexicographic: those of i < j start at first[i]
+    for (int e = 0; e < T.ne; ++e) ++first[T.edges[2 * e] + 1];
+    for (int i = 0; i < T.nn; ++i) first[i + 1] += first[i];
+    auto edge = [&](int i, int j) -> uint32_t {
+        if (i > j) std::swap(i, j);
+        int lo = first[i], hi = first[i + 1] - 1;
+        while (lo < hi) {
+            const int m = (lo + hi) / 2;
+            if (T.edges[2 * m + 1] < j) lo = m + 1;
+            else hi = m;
+        }
+        return (uint32_t)place[lo];
+    };
+    struct Inc {  // triangle t at v: (v, p, q)
+        int p, q, t;
+        bool done;
+    };
+    std::vector<int> at(T.nn + 1, 0);  // the triangles at v: inc[at[v]] .. inc[at[v + 1] - 1], by p
+    for (int v : T.tri) ++at[v + 1];
+    for (int v = 0; v < T.nn; ++v) at[v + 1] += at[v];
+    std::vector<Inc> inc(3 * (size_t)T.nt);
+    std::vector<int> fill(at.begin(), at.end() - 1);
+    for (int t = 0; t < T.nt; ++t)
+        for (int k = 0; k < 3; ++k)
+            inc[fill[T.tri[3 * t + k]]++] = {T.tri[3 * t + (k + 1) % 3], T.tri[3 * t + (k + 2) % 3], t, false};
+    std::vector<uint32_t> walk;                     // the records of all nodes
+    std::vector<size_t> begin(T.nn + 1, 0);         // of node v: walk[begin[v]] .. walk[begin[v + 1] - 1]
+    walk.reserve(4 * (3 * (size_t)T.nt + T.nn));
+    for (int v = 0; v < T.nn; ++v) {
+        Inc *lo = &inc[at[v]], *hi = &inc[0] + at[v + 1];
+        std::sort(lo, hi, [](const Inc &a, const Inc &b) { return a.p < b.p; });
+        for (Inc *f = lo; f != hi; ++f) {
+            if (f->done) continue;
+            walk.insert(walk.end(), {(uint32_t)f->p | start, edge(v, f->p), 0u, 0u});
+            // every neighbour starts exactly one triangle at v (each directed
+            // edge is used once), so the fan closes at its first neighbour
+            for (Inc *i = f; !i->done;) {
+                i->done = true;
+                walk.insert(walk.end(), {(uint32_t)i->q, edge(v, i->q), edge(i->p, i->q), (uint32_t)i->t});
+                i = std::lower_bound(lo, hi, i->q, [](const Inc &a, int key) { return a.p < key; });
+            }
+        }
+        begin[v + 1] = walk.size();
+    }
+    auto records = [&](int v) { return (begin[v + 1] - begin[v]) / 4; };
+    std::vector<int> order(T.nn);
+    for (int v = 0; v < T.nn; ++v) order[v] = v;
+    std::stable_sort(order.begin(), order.end(), [&](int a, int b) { return records(a) > records(b); });
+    T.slots.clear();
+    T.rings.clear();
+    for (int g = 0; g < T.nn; g += 32) {
+        const size_t base = T.rings.size() / 4, len = records(order[g]);
+        T.rings.resize(4 * (base + 32 * len), 0u);
+        for (int l = 0; l < 32; ++l) {
+            const int v = g + l < T.nn ? order[g + l] : -1;
+            const size_t n = v >= 0 ? records(v) : 0;
+            T.slots.insert(T.slots.end(), {v, (int)base + l, (int)n});
+            for (size_t k = 0; k < n; ++k)
+                std::copy_n(&walk[begin[v] + 4 * k], 4, &T.rings[4 * (base + 32 * k + l)]);
+        }
+    }
 }
 
 bool orient_mesh(const double *xyz, int nn, const int32_t *tris, int nt, int mode, int32_t *out, int &changed,

@@ -13,15 +13,26 @@ struct Topology {
     std::vector<double> x;                    // stretched rest coordinates [nn][3]
     std::vector<int> tri;                     // [nt][3] as given
     std::vector<int> edges;                   // [ne][2], i < j, lexicographic
+    std::vector<int> quad_tris;               // [ne][2] the triangles (a,b,c) and (d,c,b) of quad e
     std::vector<int> quads;                   // [ne][4] (a, b, c, d); edge e is (b, c) of quad e
     std::vector<double> L0, theta0, S0;       // [ne], [ne], [nt]
     double Sg0 = 0.0, V0 = 0.0;
     // device evaluation order of each element list (edges go with their
     // quads): consecutive groups of 32 elements touch pairwise-different
-    // nodes where possible, so the lanes of a warp add to different nodes'
-    // force sums
+    // nodes where possible, so the lanes of a warp load different banks
     std::vector<int> quad_order, tri_order;
+    // walks around the nodes (see ring_walks)
+    std::vector<int> slots;       // [n_slots][3]: node or -1, first record, number of records
+    std::vector<uint32_t> rings;  // [n records][4]: q | start flag, edge (v,q), edge (p,q), triangle
 };
+
+// The node pass of the membrane kernel walks the triangles (v, p, q) around
+// every node v: a starting record names the first neighbour of a fan, each
+// further one the next neighbour q, the edges (v, q) and (p, q) (numbered by
+// their place in `quad_order`) and the triangle.  Slots of 32 nodes are taken
+// by a warp: nodes come by falling number of records, and record k of the 32
+// slots lies side by side.  start: the bit that marks a starting record.
+void ring_walks(Topology &T, uint32_t start);
 
 // Evaluation order of elements (node lists of `arity` ids each) for the
 // membrane kernel, whose warps take `width` (32) consecutive elements, one
