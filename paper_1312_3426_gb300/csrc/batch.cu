@@ -34,6 +34,7 @@
 namespace lbib {
 
 constexpr int LBIB_BATCH_GRAPH_STEPS = 16;  // steps per captured graph
+constexpr int FLUID_GROUPS = 9;             // fluid kernel variants (see fluid_group)
 
 extern __shared__ float batch_smem[];
 
@@ -62,16 +63,16 @@ __global__ void __launch_bounds__(FLUID_THREADS, 5)
     fluid_block<T, BC, false>(s, (int)(t & 1), it.y * FLUID_THREADS, step_seed(t));
 }
 
-// 16-bit storage, even nx, plain boundaries: two cells per thread.
+// Even nx, plain boundaries: two cells per thread.
 template <typename T>
-__global__ void __launch_bounds__(FLUID_THREADS, 3)
+__global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>())
     k_batch_fluid_pair(const SimDev *__restrict__ sims, const long long *__restrict__ t_base, int step_off,
                        const int2 *__restrict__ items, int pf) {
-    prefetch_item<2, 2 * FLUID_THREADS>(sims, t_base, step_off, items, pf);
-    const int2 it = items[blockIdx.x];  // (simulation, block of FLUID_THREADS cell pairs)
+    prefetch_item<sizeof(T), 2 * PAIR_THREADS>(sims, t_base, step_off, items, pf);
+    const int2 it = items[blockIdx.x];  // (simulation, block of PAIR_THREADS cell pairs)
     const SimDev &s = sims[it.x];
     const long long t = t_base[it.x] + step_off;
-    const int f = 2 * (it.y * FLUID_THREADS + (int)threadIdx.x);
+    const int f = 2 * (it.y * PAIR_THREADS + (int)threadIdx.x);
     if (f < s.nf) fluid_pair<T, false>(s, (int)(t & 1), f, step_seed(t));
 }
 
@@ -126,14 +127,14 @@ struct BatchPlan {
     SimDev *d_sims = nullptr;
     long long *d_t = nullptr;
     int2 *d_items = nullptr;  // fluid (by storage type x obstacles), then node, then membrane items
-    int n_flp[8] = {};  // fluid items per kernel variant (see fluid_group)
+    int n_flp[FLUID_GROUPS] = {};  // fluid items per kernel variant (see fluid_group)
     int n_fl = 0, n_nd = 0, n_mb = 0;
     int max_nodes = 0, max_edges = 0;
     // size classes of the membrane items (largest first): the n_big items
     // within a factor 2 of the largest, and the rest, whose largest has
     // rest_nodes nodes and rest_edges edges (0: one class)
     int n_big = 0, rest_nodes = 0, rest_edges = 0;
-    int pf_cell = 0, pf_pair = 0;  // L2 prefetch distances of the fluid launches (work items)
+    int pf_cell = 0, pf_pair[2] = {};  // (pairs: 16-bit, FP32) L2 prefetch distances of the fluid launches (work items)
     cudaStream_t aux = nullptr;   // membrane kernel
     cudaStream_t aux2 = nullptr;  // membrane kernel of the smaller size class
     cudaEvent_t ev_rest = nullptr;
@@ -167,12 +168,11 @@ static BatchPlan g_plan;
 static std::mutex g_plan_mu;
 
 // Fluid kernel variant of a simulation: 2 * precision + BC (obstacles or an
-// inlet) for the one-cell-per-thread kernels; 6 / 7 for the two-cells
-// kernels of FP16 / BF16 storage (even nx, plain boundaries).
+// inlet) for the one-cell-per-thread kernels; 6 + precision for the two-cells
+// kernels.
 static int fluid_group(const lbib_sim *s) {
-    const bool bc = s->d.solid || s->d.in_on;
-    if (s->d.prec != LBIB_POP_F32 && (s->d.nx & 1) == 0 && !bc && s->d.fkern != 3) return 6 + (s->d.prec - 1);
-    return 2 * s->d.prec + (bc ? 1 : 0);
+    if (fluid_kernel_kind(s->d) != 0) return 6 + s->d.prec;
+    return 2 * s->d.prec + (s->d.solid || s->d.in_on ? 1 : 0);
 }
 
 static bool plan_matches(lbib_sim *const *sims, int n, int cluster) {
@@ -202,12 +202,12 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
         if (e == cudaSuccess) e = cudaEventCreateWithFlags(&g_plan.ev_membrane, cudaEventDisableTiming);
         if (e != cudaSuccess) return e;
     }
-    std::vector<int2> flp[8], fl, nd, mb;
+    std::vector<int2> flp[FLUID_GROUPS], fl, nd, mb;
     int max_nodes = 0, max_edges = 0;
     for (int i = 0; i < n; ++i) {
         const lbib_sim *s = sims[i];
         const int grp = fluid_group(s);
-        const int cells_per_block = grp >= 6 ? 2 * FLUID_THREADS : FLUID_THREADS;
+        const int cells_per_block = grp >= 6 ? 2 * PAIR_THREADS : FLUID_THREADS;
         const int blocks = (s->d.nf + cells_per_block - 1) / cells_per_block;
         for (int b = 0; b < blocks; ++b) flp[grp].push_back(make_int2(i, b));
         if (!s->objs.empty()) {
@@ -223,7 +223,7 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
     std::stable_sort(mb.begin(), mb.end(), [&](const int2 &a, const int2 &b) {
         return sims[a.x]->objs[a.y].nn > sims[b.x]->objs[b.y].nn;
     });
-    for (int k = 0; k < 8; ++k) {
+    for (int k = 0; k < FLUID_GROUPS; ++k) {
         g_plan.n_flp[k] = (int)flp[k].size();
         fl.insert(fl.end(), flp[k].begin(), flp[k].end());
     }
@@ -255,8 +255,9 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
     {
         int sms = 0;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g_plan.device)) != cudaSuccess) return e;
-        g_plan.pf_cell = 3 * sms / 2;  // 1.5 blocks per SM ahead (5 resident)
-        g_plan.pf_pair = sms;          // 1 block per SM ahead (3 resident)
+        g_plan.pf_cell = fluid_prefetch(LBIB_POP_F32, 0, sms);  // as in the single-simulation launches
+        g_plan.pf_pair[0] = fluid_prefetch(LBIB_POP_F16S, 1, sms);
+        g_plan.pf_pair[1] = fluid_prefetch(LBIB_POP_F32, 1, sms);
     }
     g_plan.max_nodes = max_nodes;
     g_plan.max_edges = max_edges;
@@ -367,8 +368,7 @@ static cudaError_t enqueue_steps(cudaStream_t st, int step_off, int k) {
             const int *n = g_plan.n_flp;
             const SimDev *ds = g_plan.d_sims;
             const long long *dt = g_plan.d_t;
-            // prefetch distances as in the single-simulation launches
-            const int p1 = g_plan.pf_cell, p2 = g_plan.pf_pair;
+            const int p1 = g_plan.pf_cell, p2 = g_plan.pf_pair[0], p4 = g_plan.pf_pair[1];
             if (n[0]) k_batch_fluid<float, false><<<n[0], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p1);
             g += n[0];
             if (n[1]) k_batch_fluid<float, true><<<n[1], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p1);
@@ -381,9 +381,11 @@ static cudaError_t enqueue_steps(cudaStream_t st, int step_off, int k) {
             g += n[4];
             if (n[5]) k_batch_fluid<__nv_bfloat16, true><<<n[5], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p1);
             g += n[5];
-            if (n[6]) k_batch_fluid_pair<__half><<<n[6], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p2);
+            if (n[6]) k_batch_fluid_pair<float><<<n[6], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p4);
             g += n[6];
-            if (n[7]) k_batch_fluid_pair<__nv_bfloat16><<<n[7], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p2);
+            if (n[7]) k_batch_fluid_pair<__half><<<n[7], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
+            g += n[7];
+            if (n[8]) k_batch_fluid_pair<__nv_bfloat16><<<n[8], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if (g_plan.n_nd) e = cudaStreamWaitEvent(st, g_plan.ev_membrane, 0);

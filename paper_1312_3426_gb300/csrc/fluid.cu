@@ -1,7 +1,8 @@
 // Fluid kernels: fused pull-stream + collide (Eq. lbequation), read-outs,
 // checkpoint conversion and the FP64 mass reduction.
 //
-// One thread updates one fluid cell.  For each of the 19 directions it pulls
+// One thread updates one fluid cell, or two x-adjacent ones where nx is even
+// and there are no obstacles and no inlet.  For each of the 19 directions it pulls
 // the post-collision value of the previous step from the neighbour the
 // population comes from (periodic in x and z, and in y without walls); a
 // population that would come from a solid row is the cell's own opposite
@@ -19,6 +20,7 @@
 // touched by the immersed objects.
 #include <mutex>
 #include <type_traits>
+#include <utility>
 
 #include "fluid_core.cuh"
 
@@ -26,20 +28,24 @@ namespace lbib {
 
 // EARLY: the instantiation for an early (programmatic dependent) launch
 template <typename T, bool BC, bool EARLY>
-__global__ void __launch_bounds__(FLUID_THREADS, 5) k_fluid(SimDev s, int par, uint32_t seed, int pf) {
-    prefetch_sources<sizeof(T), FLUID_THREADS>(s, s.pop[par], pf);
-    fluid_block<T, BC, EARLY>(s, par, blockIdx.x * FLUID_THREADS, seed);
+__global__ void __launch_bounds__(FLUID_THREADS, 5) k_fluid(SimDev s, uint32_t seed, int pf) {
+    prefetch_sources<sizeof(T), FLUID_THREADS>(s, s.pop[0], pf);
+    fluid_block<T, BC, EARLY>(s, 0, blockIdx.x * FLUID_THREADS, seed);
 }
 
-// 16-bit storage, even nx, no obstacles, no inlet: two cells per thread.
-// Blocks of 128 threads (6 per SM at 80 registers): when a membrane block
-// shares the SM, one of six fluid blocks gives way instead of one of three.
-constexpr int PAIR_THREADS = 128;
+// Even nx, no obstacles, no inlet: two cells per thread.  Both cells share
+// the index work and the packed FP32 instructions, so a warp of 64 cells
+// issues 557 (FP32) or 596 (16-bit) instructions; one cell per thread took
+// 651 for 32 FP32 cells.  FP32 is bound by DRAM either way (256x128x128
+// without objects 95.4 -> 94.3 us a step, 6.7 TB/s; 35.9 M instead of 84.0 M
+// warp instructions, which leaves the issue slots to the membrane kernel
+// beside it), the 16-bit kernel by instructions (61.6 -> 57.6 us there and
+// 455 -> 431 at 512x256x256, 47.1 -> 38.4 M).
 template <typename T, bool EARLY>
-__global__ void __launch_bounds__(PAIR_THREADS, 6) k_fluid_pair(SimDev s, int par, uint32_t seed, int pf) {
-    prefetch_sources<2, 2 * PAIR_THREADS>(s, s.pop[par], pf);
+__global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>()) k_fluid_pair(SimDev s, uint32_t seed, int pf) {
+    prefetch_sources<sizeof(T), 2 * PAIR_THREADS>(s, s.pop[0], pf);
     const int f = 2 * (int)(blockIdx.x * PAIR_THREADS + threadIdx.x);
-    if (f < s.nf) fluid_pair<T, EARLY>(s, par, f, seed);
+    if (f < s.nf) fluid_pair<T, EARLY>(s, 0, f, seed);
 }
 
 static bool pair_shape(const SimDev &s) { return (s.nx & 1) == 0 && !s.solid && !s.in_on; }
@@ -49,7 +55,8 @@ static bool pair_shape(const SimDev &s) { return (s.nx & 1) == 0 && !s.solid && 
 // vs 0.0882 ms in the step at 256x128x128, 0.764 vs 0.709 ms at
 // 512x256x256) and slowed the membrane kernel beside it.
 int fluid_kernel_kind(const SimDev &s) {
-    if (s.prec == LBIB_POP_F32 || !pair_shape(s) || s.fkern == 3) return 0;
+    if (!pair_shape(s) || (s.prec != LBIB_POP_F32 && s.fkern == 3)) return 0;
+    if (s.prec == LBIB_POP_F32) return 1;
     if (s.fkern == 2 && fluid_tma_shape(s)) return 2;
     return 1;
 }
@@ -64,32 +71,42 @@ int device_sms() {
     return sms[dev];
 }
 
-// Prefetch distances (in blocks), measured at 256x128x128 and 512x256x256
-// on a GB300: 1.5 blocks per SM ahead for the one-cell kernel (5 resident
-// per SM), 3 per SM for the two-cells kernel (6 resident per SM).
+// Measured at 256x128x128 and 512x256x256 on a GB300: 1.5 blocks per SM ahead
+// for the one-cell kernel (5 blocks of 256 resident per SM) and the FP32
+// two-cells kernel (5 blocks of 128; 94.3 against 95.2 us for 3 per SM), 3 per
+// SM for the 16-bit two-cells kernel (6 of 128; 59.7 against 61.3 for 1.5).
+int fluid_prefetch(int prec, int kind, int sms) { return kind == 1 && prec != LBIB_POP_F32 ? 3 * sms : 3 * sms / 2; }
+
 // pdl: the warp-specialised kernel is always launched plainly.
 template <typename T>
 static cudaError_t launch_fluid_t(const SimDev &s, int par, uint32_t seed, int blocks, cudaStream_t st, bool pdl) {
     const int sms = device_sms();
-    if constexpr (sizeof(T) == 2) {
-        if (fluid_kernel_kind(s) == 2) {
-            launch_fluid_tma(s, par, seed, st);
-            return cudaGetLastError();
-        }
-        if (fluid_kernel_kind(s) == 1) {
-            const unsigned pblocks = (unsigned)((s.nf / 2 + PAIR_THREADS - 1) / PAIR_THREADS);
-            if (pdl) return launch_dep(k_fluid_pair<T, true>, pblocks, PAIR_THREADS, st, true, s, par, seed, 3 * sms);
-            return launch_dep(k_fluid_pair<T, false>, pblocks, PAIR_THREADS, st, false, s, par, seed, 3 * sms);
-        }
+    if (fluid_kernel_kind(s) == 2) {
+        launch_fluid_tma(s, par, seed, st);
+        return cudaGetLastError();
+    }
+    // The kernels take the buffers in the order source, destination, so that
+    // a plane's base is the same computation for all threads (uniform
+    // registers) instead of a load at an index that the step decides.
+    SimDev d = s;
+    if (par) {
+        std::swap(d.pop[0], d.pop[1]);
+        std::swap(d.G[0], d.G[1]);
+    }
+    if (fluid_kernel_kind(s) == 1) {
+        const unsigned pblocks = (unsigned)((s.nf / 2 + PAIR_THREADS - 1) / PAIR_THREADS);
+        const int pf = fluid_prefetch(s.prec, 1, sms);
+        if (pdl) return launch_dep(k_fluid_pair<T, true>, pblocks, PAIR_THREADS, st, true, d, seed, pf);
+        return launch_dep(k_fluid_pair<T, false>, pblocks, PAIR_THREADS, st, false, d, seed, pf);
     }
     const unsigned b = (unsigned)blocks;
-    const int pf = 3 * sms / 2;
+    const int pf = fluid_prefetch(s.prec, 0, sms);
     if (s.solid || s.in_on) {
-        if (pdl) return launch_dep(k_fluid<T, true, true>, b, FLUID_THREADS, st, true, s, par, seed, pf);
-        return launch_dep(k_fluid<T, true, false>, b, FLUID_THREADS, st, false, s, par, seed, pf);
+        if (pdl) return launch_dep(k_fluid<T, true, true>, b, FLUID_THREADS, st, true, d, seed, pf);
+        return launch_dep(k_fluid<T, true, false>, b, FLUID_THREADS, st, false, d, seed, pf);
     }
-    if (pdl) return launch_dep(k_fluid<T, false, true>, b, FLUID_THREADS, st, true, s, par, seed, pf);
-    return launch_dep(k_fluid<T, false, false>, b, FLUID_THREADS, st, false, s, par, seed, pf);
+    if (pdl) return launch_dep(k_fluid<T, false, true>, b, FLUID_THREADS, st, true, d, seed, pf);
+    return launch_dep(k_fluid<T, false, false>, b, FLUID_THREADS, st, false, d, seed, pf);
 }
 
 cudaError_t launch_fluid(const SimDev &s, int par, long long t, cudaStream_t st, bool pdl) {

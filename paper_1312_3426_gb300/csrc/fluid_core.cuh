@@ -53,29 +53,23 @@ __device__ __forceinline__ uint32_t mix32(uint32_t x) {
     return x;
 }
 
-// Neighbour offsets of one cell in the fluid index space.
-struct Nbr {
-    int dxm, dxp, dym, dyp, dzm, dzp;  // index delta to the cell at x-1, x+1, ...
-    bool ylo_solid, yhi_solid;         // the row below / above is a wall
+// Where a cell (or the first cell of a pair) pulls from, as indices into a
+// plane (a plane's base is the same for all threads, so an address is one
+// multiply-add of a 32-bit index): the rows (y - ey, z - ez), all axes
+// periodic.
+struct Rows {
+    uint32_t row[3][3];  // [1 + ey][1 + ez], at the cell's own x
 };
-
-__device__ __forceinline__ Nbr neighbours(const SimDev &s, int x, int y, int z) {
-    Nbr n;
-    const int plane = s.nx * s.nyf;
-    n.dxm = (x == 0) ? s.nx - 1 : -1;
-    n.dxp = (x == s.nx - 1) ? -(s.nx - 1) : 1;
-    n.dzm = (z == 0) ? (s.nz - 1) * plane : -plane;
-    n.dzp = (z == s.nz - 1) ? -(s.nz - 1) * plane : plane;
-    if (s.walls) {
-        n.ylo_solid = (y == 0);
-        n.yhi_solid = (y == s.nyf - 1);
-        n.dym = -s.nx;
-        n.dyp = s.nx;
-    } else {
-        n.ylo_solid = n.yhi_solid = false;
-        n.dym = (y == 0) ? (s.nyf - 1) * s.nx : -s.nx;
-        n.dyp = (y == s.nyf - 1) ? -(s.nyf - 1) * s.nx : s.nx;
-    }
+__device__ __forceinline__ Rows source_rows(const SimDev &s, uint32_t f, int y, int z) {
+    Rows n;
+    const int ry = s.nx, rz = s.nx * s.nyf;
+    const int ym = y == 0 ? (s.nyf - 1) * ry : -ry, yp = y == s.nyf - 1 ? -(s.nyf - 1) * ry : ry;
+    const int zm = z == 0 ? (s.nz - 1) * rz : -rz, zp = z == s.nz - 1 ? -(s.nz - 1) * rz : rz;
+    const int dy[3] = {yp, 0, ym}, dz[3] = {zp, 0, zm};
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) n.row[i][j] = f + (uint32_t)(dy[i] + dz[j]);
     return n;
 }
 
@@ -135,24 +129,31 @@ struct Raw<__nv_bfloat16> {
     }
 };
 
-// Pull the (raw) population of direction Q arriving at cell f.  In the
+// Pull the (raw) population of direction Q arriving at a cell (xm, xp: steps
+// to x - 1 and x + 1, periodic; walls not considered).  In the
 // boundary-condition variant (BC) a population coming from an obstacle cell
 // is the cell's own opposite one, as at the walls.
 template <typename T, int Q, bool BC>
-__device__ __forceinline__ float pull(const SimDev &s, const T *__restrict__ src, uint32_t nfp, uint32_t f,
-                                      const Nbr &n) {
+__device__ __forceinline__ float pull(const SimDev &s, const T *__restrict__ src, size_t nfp, const Rows &n, int xm,
+                                      int xp) {
     constexpr int ex = d3q19_ex(Q), ey = d3q19_ey(Q), ez = d3q19_ez(Q);
-    if ((ey == 1 && n.ylo_solid) || (ey == -1 && n.yhi_solid))
-        return Raw<T>::ld(src + (uint32_t)d3q19_opp(Q) * nfp + f);
-    int g = (int)f;
-    if (ex == 1) g += n.dxm;
-    if (ex == -1) g += n.dxp;
-    if (ey == 1) g += n.dym;
-    if (ey == -1) g += n.dyp;
-    if (ez == 1) g += n.dzm;
-    if (ez == -1) g += n.dzp;
-    if (BC && Q != 0 && s.solid && solid_bit(s, g)) return Raw<T>::ld(src + (uint32_t)d3q19_opp(Q) * nfp + f);
-    return Raw<T>::ld(src + (uint32_t)Q * nfp + (uint32_t)g);
+    uint32_t g = n.row[1 + ey][1 + ez];
+    if constexpr (ex == 1) g += (uint32_t)xm;
+    if constexpr (ex == -1) g += (uint32_t)xp;
+    if (BC && Q != 0 && s.solid && solid_bit(s, (int)g))
+        return Raw<T>::ld(src + (size_t)d3q19_opp(Q) * nfp + n.row[1][1]);
+    return Raw<T>::ld(src + (size_t)Q * nfp + g);
+}
+
+// Bounce-back at a wall row (the row below, EY = 1, or above, EY = -1, is
+// solid): the populations with that ey are the cell's own opposite ones.
+// Their periodic pulls, already on the way, are replaced; only warps with a
+// cell of a wall row come here.
+template <typename T, int EY>
+__device__ __forceinline__ void bounce(const T *__restrict__ src, size_t nfp, uint32_t f, float (&h)[NQ]) {
+#pragma unroll
+    for (int q = 1; q < NQ; ++q)
+        if (d3q19_ey(q) == EY) h[q] = Raw<T>::ld(src + (size_t)d3q19_opp(q) * nfp + f);
 }
 
 // BGK + Guo update of the opposite pair (Q, Q+1) (e_{Q+1} = -e_Q, same
@@ -435,14 +436,20 @@ __device__ __forceinline__ void fluid_cell(const SimDev &s, int par, int fi, uin
     const uint32_t x = f - r * (uint32_t)s.nx;
     const uint32_t z = s.div_nyf.div(r);
     const uint32_t y = r - z * (uint32_t)s.nyf;
-    const Nbr n = neighbours(s, (int)x, (int)y, (int)z);
+    const Rows n = source_rows(s, f, (int)y, (int)z);
+    const int xm = x == 0 ? s.nx - 1 : -1, xp = x == (uint32_t)s.nx - 1 ? 1 - s.nx : 1;
 
     float h[NQ];
-#define LBIB_PULL(q) h[q] = pull<T, q, BC>(s, src, nfp, f, n);
+#define LBIB_PULL(q) h[q] = pull<T, q, BC>(s, src, nfp, n, xm, xp);
     LBIB_PULL(0) LBIB_PULL(1) LBIB_PULL(2) LBIB_PULL(3) LBIB_PULL(4) LBIB_PULL(5) LBIB_PULL(6)
     LBIB_PULL(7) LBIB_PULL(8) LBIB_PULL(9) LBIB_PULL(10) LBIB_PULL(11) LBIB_PULL(12) LBIB_PULL(13)
     LBIB_PULL(14) LBIB_PULL(15) LBIB_PULL(16) LBIB_PULL(17) LBIB_PULL(18)
 #undef LBIB_PULL
+    const bool ylo = s.walls && y == 0, yhi = s.walls && y == (uint32_t)s.nyf - 1;
+    if (__any_sync(__activemask(), ylo || yhi)) {
+        if (ylo) bounce<T, 1>(src, nfp, f, h);
+        if (yhi) bounce<T, -1>(src, nfp, f, h);
+    }
 
     if (BC && s.in_on) inlet_cell(s, (int)x, (int)y + s.walls, (int)z, h);
     // the populations pulled above were written by the previous fluid step;
@@ -455,7 +462,10 @@ __device__ __forceinline__ void fluid_cell(const SimDev &s, int par, int fi, uin
     const bool active = (act >> (fi & 31)) & 1u;
 
     float Gx = s.gx, Gy = s.gy, Gz = s.gz;
-    if (active) {  // spread force of this step; clear the buffer of the next
+    // spread force of this step; clear the buffer of the next.  Most warps have
+    // no active cell: a warp vote keeps this behind a branch (a plain
+    // condition becomes predicated instructions that every warp issues).
+    if (__any_sync(__activemask(), active) && active) {
         const float4 g = __ldcg(s.G[par] + f);
         Gx += g.x;
         Gy += g.y;
@@ -534,32 +544,60 @@ struct Half2Bits<__nv_bfloat16> {
     static __device__ __forceinline__ float hi(uint32_t u) { return __uint_as_float(u & 0xffff0000u); }
 };
 
-// The pair of direction Q arriving at cells f, f+1 (low half: cell f).
-// dxm0: x-1 offset of cell f (wraps at x = 0); dxp1: x+1 offset of cell f+1
-// (wraps at x+1 = nx-1).  Marking these loads evict-first in L2 kept the
-// velocity and force fields for the node update that follows (20.7 -> 18.2
-// us at 256x128x128) but slowed the kernel 6% at 512x256x256, where the
-// x-shifted lines shared by neighbouring warps were evicted in between; the
-// loads keep the default policy.
-template <int Q>
-__device__ __forceinline__ uint32_t pull2(const uint16_t *__restrict__ src, uint32_t nfp, uint32_t f, const Nbr &n,
-                                          int dxm0, int dxp1) {
+// Blocks of 128 threads: when a membrane block shares the SM, one of five or
+// six fluid blocks gives way instead of one of three.
+constexpr int PAIR_THREADS = 128;
+template <typename T>
+constexpr int pair_blocks() {  // per SM, at 96 (FP32) and 80 registers a thread
+    return sizeof(T) == 4 ? 5 : 6;
+}
+
+// A stored pair of cells: two 16-bit numbers in a word (low half: cell f), or
+// two FP32 numbers; p[i], p[i + 1] (i even) or p[i], p[j].
+template <typename T>
+struct PairRaw {
+    using type = uint32_t;
+    static __device__ __forceinline__ uint32_t ld(const T *p, uint32_t i) {
+        return __ldg((const unsigned int *)(p + i));
+    }
+    static __device__ __forceinline__ uint32_t ld(const T *p, uint32_t i, uint32_t j) {
+        return (uint32_t)__ldg((const unsigned short *)p + i) | ((uint32_t)__ldg((const unsigned short *)p + j) << 16);
+    }
+};
+template <>
+struct PairRaw<float> {
+    using type = float2;
+    static __device__ __forceinline__ float2 ld(const float *p, uint32_t i) { return __ldg((const float2 *)(p + i)); }
+    static __device__ __forceinline__ float2 ld(const float *p, uint32_t i, uint32_t j) {
+        return make_float2(__ldg(p + i), __ldg(p + j));
+    }
+};
+
+// The pair of direction Q arriving at cells f, f+1 (xm, xp: steps from f to
+// x - 1 and to x + 2, periodic; walls not considered).
+// Marking these loads evict-first in L2 kept the velocity and force fields
+// for the node update that follows (20.7 -> 18.2 us at 256x128x128) but
+// slowed the kernel 6% at 512x256x256, where the x-shifted lines shared by
+// neighbouring warps were evicted in between; the loads keep the default
+// policy.
+template <typename T, int Q>
+__device__ __forceinline__ typename PairRaw<T>::type pull2(const T *__restrict__ src, size_t nfp, const Rows &n, int xm,
+                                                           int xp) {
     constexpr int ex = d3q19_ex(Q), ey = d3q19_ey(Q), ez = d3q19_ez(Q);
-    if ((ey == 1 && n.ylo_solid) || (ey == -1 && n.yhi_solid))
-        return __ldg((const unsigned int *)(src + (uint32_t)d3q19_opp(Q) * nfp + f));
-    int g = (int)f;
-    if (ey == 1) g += n.dym;
-    if (ey == -1) g += n.dyp;
-    if (ez == 1) g += n.dzm;
-    if (ez == -1) g += n.dzp;
-    const uint16_t *p = src + (uint32_t)Q * nfp;
-    if (ex == 0) return __ldg((const unsigned int *)(p + (uint32_t)g));  // g even
-    if (ex == 1)  // cell f from x-1, cell f+1 from x
-        return (uint32_t)__ldg((const unsigned short *)(p + (uint32_t)(g + dxm0))) |
-               ((uint32_t)__ldg((const unsigned short *)(p + (uint32_t)g)) << 16);
-    // ex == -1: cell f from x+1, cell f+1 from x+2 (or the row start)
-    return (uint32_t)__ldg((const unsigned short *)(p + (uint32_t)(g + 1))) |
-           ((uint32_t)__ldg((const unsigned short *)(p + (uint32_t)(g + 1 + dxp1))) << 16);
+    const T *p = src + (size_t)Q * nfp;
+    const uint32_t o = n.row[1 + ey][1 + ez];
+    if constexpr (ex == 0) return PairRaw<T>::ld(p, o);
+    else if constexpr (ex == 1) return PairRaw<T>::ld(p, o + (uint32_t)xm, o);  // from x - 1 and x
+    else return PairRaw<T>::ld(p, o + 1u, o + (uint32_t)xp);                    // from x + 1 and x + 2
+}
+
+// bounce() of the pair
+template <typename T, int EY>
+__device__ __forceinline__ void bounce2(const T *__restrict__ src, size_t nfp, uint32_t f,
+                                        typename PairRaw<T>::type (&P)[NQ]) {
+#pragma unroll
+    for (int q = 1; q < NQ; ++q)
+        if (d3q19_ey(q) == EY) P[q] = PairRaw<T>::ld(src + (size_t)d3q19_opp(q) * nfp, f);
 }
 
 // The arithmetic of the two cells runs in packed FP32 instructions (sm_100
@@ -606,6 +644,13 @@ __device__ __forceinline__ float2 unpack2(uint32_t u) {
     return make_float2(Half2Bits<T>::lo(u), Half2Bits<T>::hi(u));
 }
 
+// The pair as two FP32 numbers
+template <typename T>
+__device__ __forceinline__ float2 pair_f32(typename PairRaw<T>::type v) {
+    if constexpr (sizeof(T) == 4) return v;
+    else return unpack2<T>(v);
+}
+
 struct Moments2 {
     float2 r, x, y, z;
 };
@@ -619,20 +664,20 @@ __device__ __forceinline__ void add_diff2(Moments2 &m, float2 d) {
 // The moments of both cells: sum h from the pair sums, sum h e from the
 // pair differences; the axis pairs (1, 3, 5) open the x, y, z sums.
 template <typename T>
-__device__ __forceinline__ Moments2 moments2(const uint32_t (&P)[NQ]) {
+__device__ __forceinline__ Moments2 moments2(const typename PairRaw<T>::type (&P)[NQ]) {
     static_assert(d3q19_ex(1) == 1 && d3q19_ey(3) == 1 && d3q19_ez(5) == 1, "axis pairs 1, 3, 5");
     Moments2 m;
-    float2 a = unpack2<T>(P[1]), b = unpack2<T>(P[2]);
-    m.r = add2(unpack2<T>(P[0]), add2(a, b));
+    float2 a = pair_f32<T>(P[1]), b = pair_f32<T>(P[2]);
+    m.r = add2(pair_f32<T>(P[0]), add2(a, b));
     m.x = sub2(a, b);
-    a = unpack2<T>(P[3]), b = unpack2<T>(P[4]);
+    a = pair_f32<T>(P[3]), b = pair_f32<T>(P[4]);
     m.r = add2(m.r, add2(a, b));
     m.y = sub2(a, b);
-    a = unpack2<T>(P[5]), b = unpack2<T>(P[6]);
+    a = pair_f32<T>(P[5]), b = pair_f32<T>(P[6]);
     m.r = add2(m.r, add2(a, b));
     m.z = sub2(a, b);
 #define LBIB_M2(q)                          \
-    a = unpack2<T>(P[q]), b = unpack2<T>(P[q + 1]); \
+    a = pair_f32<T>(P[q]), b = pair_f32<T>(P[q + 1]); \
     m.r = add2(m.r, add2(a, b));            \
     add_diff2<q>(m, sub2(a, b));
     LBIB_M2(7) LBIB_M2(9) LBIB_M2(11) LBIB_M2(13) LBIB_M2(15) LBIB_M2(17)
@@ -688,8 +733,8 @@ __device__ __forceinline__ void pair_terms2(const Coll2 &c, const Cls2 &w, float
 }
 
 template <typename T, int Q>
-__device__ __forceinline__ void collide2(uint32_t *__restrict__ dst, uint32_t nfp2, uint32_t f2, uint32_t Pq,
-                                         uint32_t Po, const Coll2 &c, const CollK &k, const Cls2 &w,
+__device__ __forceinline__ void collide2(uint16_t *__restrict__ dst, size_t nfp, uint32_t f, uint32_t Pq, uint32_t Po,
+                                         const Coll2 &c, const CollK &k, const Cls2 &w,
                                          uint32_t &rng) {
     float2 ApB, AmB;
     pair_terms2<Q>(c, w, ApB, AmB);
@@ -702,76 +747,161 @@ __device__ __forceinline__ void collide2(uint32_t *__restrict__ dst, uint32_t nf
     // changes the variance of sums over two cells, not their mean (the
     // 16-bit Poiseuille errors were unchanged: 2.66e-4 FP16, 1.52e-3 BF16).
     const uint32_t r2 = __byte_perm(r1, 0u, 0x1032);
-    __stcs((unsigned int *)(dst + (uint32_t)Q * nfp2 + f2), Pack2<T>::rs(oq.x, oq.y, r1));
-    __stcs((unsigned int *)(dst + (uint32_t)(Q + 1) * nfp2 + f2), Pack2<T>::rs(oo.x, oo.y, r2));
+    __stcs((unsigned int *)(dst + (size_t)Q * nfp + f), Pack2<T>::rs(oq.x, oq.y, r1));
+    __stcs((unsigned int *)(dst + (size_t)(Q + 1) * nfp + f), Pack2<T>::rs(oo.x, oo.y, r2));
+}
+
+// The increment form (struct Inc) of both FP32 cells, in packed instructions:
+// the same parts per opposite pair, with the products of constants and cell
+// quantities that a weight class shares formed once.
+struct Inc2 {
+    Moments2 m;               // j in x, y, z
+    float2 ux, uy, uz, Gx, Gy, Gz, m3uG;
+    float om;
+};
+struct IncCls2 {
+    float2 r45, K;            // w (4.5 rho), w K
+    float chi, clo, fw;       // 3 w as hi + lo, fpre w
+};
+template <int Q>
+__device__ __forceinline__ void inc_pair2(float *__restrict__ dst, size_t nfp, uint32_t f, float2 hq, float2 ho,
+                                          const Inc2 &c, const IncCls2 &w) {
+    const float2 ej = edot2<Q>(c.m.x, c.m.y, c.m.z), eu = edot2<Q>(c.ux, c.uy, c.uz), eG = edot2<Q>(c.Gx, c.Gy, c.Gz);
+    float2 t = fma2(v2(w.chi), ej, mul2(v2(-0.5f), sub2(hq, ho)));
+    t = fma2(v2(w.clo), ej, t);
+    const float2 Do = fma2(v2(c.om), t, fma2(v2(w.chi), eG, mul2(v2(w.clo), eG)));
+    const float2 Aeq = fma2(w.r45, mul2(eu, eu), w.K);
+    const float2 Fe = mul2(v2(w.fw), fma2(mul2(v2(9.0f), eu), eG, c.m3uG));
+    const float2 De = fma2(v2(c.om), fma2(v2(-0.5f), add2(hq, ho), Aeq), Fe);
+    __stcs((float2 *)(dst + (size_t)Q * nfp + f), add2(hq, add2(De, Do)));
+    __stcs((float2 *)(dst + (size_t)(Q + 1) * nfp + f), add2(ho, sub2(De, Do)));
+}
+
+// Collision and store of the FP32 pair; sets u, rho and returns u.u.
+__device__ __forceinline__ float2 collide_increment2(const SimDev &s, float *__restrict__ dst, size_t nfp, uint32_t f,
+                                                     const float2 (&h)[NQ], Inc2 &c, float2 &rho) {
+    c.m = moments2<float>(h);
+    c.om = s.omega;
+    rho = add2(v2(s.rho0), c.m.r);
+    // rho is near 1: the fast reciprocal is within 2 ulp
+    const float2 irho = make_float2(__fdividef(1.0f, rho.x), __fdividef(1.0f, rho.y));
+    c.ux = mul2(fma2(v2(0.5f), c.Gx, c.m.x), irho);
+    c.uy = mul2(fma2(v2(0.5f), c.Gy, c.m.y), irho);
+    c.uz = mul2(fma2(v2(0.5f), c.Gz, c.m.z), irho);
+    const float2 usq = fma2(c.uz, c.uz, fma2(c.uy, c.uy, mul2(c.ux, c.ux)));
+    c.m3uG = mul2(v2(-3.0f), fma2(c.uz, c.Gz, fma2(c.uy, c.Gy, mul2(c.ux, c.Gx))));
+    const float2 K = fma2(mul2(v2(-1.5f), rho), usq, c.m.r), r45 = mul2(v2(4.5f), rho);
+    constexpr float w0 = (float)(1.0 / 3.0), w1 = (float)(1.0 / 18.0), w2 = (float)(1.0 / 36.0);
+    __stcs((float2 *)(dst + f),
+           add2(h[0], fma2(v2(c.om), fma2(v2(w0), K, mul2(v2(-1.0f), h[0])), mul2(v2(s.fpre * w0), c.m3uG))));
+    {
+        const IncCls2 w{mul2(r45, v2(w1)), mul2(v2(w1), K), INC_C1_HI, INC_C1_LO, s.fpre * w1};
+        inc_pair2<1>(dst, nfp, f, h[1], h[2], c, w);
+        inc_pair2<3>(dst, nfp, f, h[3], h[4], c, w);
+        inc_pair2<5>(dst, nfp, f, h[5], h[6], c, w);
+    }
+    const IncCls2 w{mul2(r45, v2(w2)), mul2(v2(w2), K), 0.5f * INC_C1_HI, 0.5f * INC_C1_LO, s.fpre * w2};
+    inc_pair2<7>(dst, nfp, f, h[7], h[8], c, w);
+    inc_pair2<9>(dst, nfp, f, h[9], h[10], c, w);
+    inc_pair2<11>(dst, nfp, f, h[11], h[12], c, w);
+    inc_pair2<13>(dst, nfp, f, h[13], h[14], c, w);
+    inc_pair2<15>(dst, nfp, f, h[15], h[16], c, w);
+    inc_pair2<17>(dst, nfp, f, h[17], h[18], c, w);
+    return usq;
 }
 
 // Collision and store of the cell pair (f, f+1) from its pulled populations
 // P (packed pairs, low half: cell f).
-// act: the active-cell bits of f (bit 0) and f + 1 (bit 1).
-template <typename T>
-__device__ __forceinline__ void pair_update_act(const SimDev &s, int par, uint32_t f, const uint32_t (&P)[NQ],
-                                                uint32_t step_seed, uint32_t act) {
-    uint32_t *__restrict__ dst = (uint32_t *)s.pop[par ^ 1];
-    const uint32_t nfp = (uint32_t)s.nfp;
-    float4 ga = make_float4(0.f, 0.f, 0.f, 0.f), gb = ga;
-    if (act & 1u) {  // spread force of this step; clear the buffer of the next
-        ga = __ldcg(s.G[par] + f);
-        s.G[par ^ 1][f] = make_float4(0.f, 0.f, 0.f, 0.f);
+// c: the coupling of the pair, as load_coupling returned it.
+struct Coupling {
+    float4 a, b;   // spread force on cells f and f + 1
+    uint32_t act;  // active-cell bits of f (bit 0) and f + 1 (bit 1)
+    bool any;      // of the warp
+};
+// The spread force of this step on the active cells of the pair; clears
+// their places in the buffer of the next.  Most warps have no active cell: a
+// warp vote keeps the rest behind a branch (a plain condition becomes
+// predicated instructions that every warp issues).  Issuing these loads
+// right after the pulls', before their first use, was no faster with objects
+// (67.7 us for the 16-bit kernel at 256x128x128 with 200 cells either way)
+// and slower without (59.2 against 57.6).
+__device__ __forceinline__ Coupling load_coupling(const SimDev &s, int par, uint32_t f, uint32_t act) {
+    Coupling c{make_float4(0.f, 0.f, 0.f, 0.f), make_float4(0.f, 0.f, 0.f, 0.f), act,
+               (bool)__any_sync(__activemask(), act != 0u)};
+    if (c.any) {
+        if (act & 1u) c.a = __ldcg(s.G[par] + f);
+        if (act & 2u) c.b = __ldcg(s.G[par] + f + 1);
+        if (act & 1u) s.G[par ^ 1][f] = make_float4(0.f, 0.f, 0.f, 0.f);
+        if (act & 2u) s.G[par ^ 1][f + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
     }
-    if (act & 2u) {
-        gb = __ldcg(s.G[par] + f + 1);
-        s.G[par ^ 1][f + 1] = make_float4(0.f, 0.f, 0.f, 0.f);
-    }
-    const CollK k = make_collk(s);
-    float2 rho, usq;
-    const Moments2 m = moments2<T>(P);
-    const Coll2 c = make_coll2(s, k, m, make_float2(s.gx + ga.x, s.gx + gb.x), make_float2(s.gy + ga.y, s.gy + gb.y),
-                               make_float2(s.gz + ga.z, s.gz + gb.z), rho, usq);
-    const float sc = s.scale;
-    const float wsc0 = (float)d3q19_w(0) * sc, wsc1 = (float)d3q19_w(1) * sc, wsc2 = (float)d3q19_w(7) * sc;
-    const uint32_t nfp2 = nfp / 2, f2 = f / 2;
-    uint32_t rng = mix32(f ^ step_seed);
-    rng = rng * 747796405u + 2891336453u;
-    const float2 o0 = fma2(v2(k.c1), unpack2<T>(P[0]), mul2(v2(wsc0), c.Kb));
-    __stcs((unsigned int *)(dst + f2), Pack2<T>::rs(o0.x, o0.y, rng ^ (rng >> 15)));
-    {
-        const Cls2 w = make_cls2(c, k, wsc1);
-        collide2<T, 1>(dst, nfp2, f2, P[1], P[2], c, k, w, rng);
-        collide2<T, 3>(dst, nfp2, f2, P[3], P[4], c, k, w, rng);
-        collide2<T, 5>(dst, nfp2, f2, P[5], P[6], c, k, w, rng);
-    }
-    const Cls2 w = make_cls2(c, k, wsc2);
-    collide2<T, 7>(dst, nfp2, f2, P[7], P[8], c, k, w, rng);
-    collide2<T, 9>(dst, nfp2, f2, P[9], P[10], c, k, w, rng);
-    collide2<T, 11>(dst, nfp2, f2, P[11], P[12], c, k, w, rng);
-    collide2<T, 13>(dst, nfp2, f2, P[13], P[14], c, k, w, rng);
-    collide2<T, 15>(dst, nfp2, f2, P[15], P[16], c, k, w, rng);
-    collide2<T, 17>(dst, nfp2, f2, P[17], P[18], c, k, w, rng);
-    if (act & 1u) s.ufield[f] = make_float4(c.ux.x, c.uy.x, c.uz.x, rho.x);
-    if (act & 2u) s.ufield[f + 1] = make_float4(c.ux.y, c.uy.y, c.uz.y, rho.y);
-    if (!(usq.x < 0.09f) || !(usq.y < 0.09f)) atomicOr(s.status, ST_UNSTABLE);
+    return c;
 }
 
 template <typename T>
-__device__ __forceinline__ void pair_update(const SimDev &s, int par, uint32_t f, const uint32_t (&P)[NQ],
-                                            uint32_t step_seed) {
-    pair_update_act<T>(s, par, f, P, step_seed, (__ldcg(s.amask + (f >> 5)) >> (f & 31)) & 3u);
+__device__ __forceinline__ void pair_update(const SimDev &s, int par, uint32_t f, const typename PairRaw<T>::type (&P)[NQ],
+                                            uint32_t step_seed, const Coupling &cp) {
+    const size_t nfp = (size_t)s.nfp;
+    const float2 Gx = make_float2(s.gx + cp.a.x, s.gx + cp.b.x), Gy = make_float2(s.gy + cp.a.y, s.gy + cp.b.y),
+                 Gz = make_float2(s.gz + cp.a.z, s.gz + cp.b.z);
+    float2 rho, usq, ux, uy, uz;
+    if constexpr (sizeof(T) == 4) {
+        Inc2 c;
+        c.Gx = Gx;
+        c.Gy = Gy;
+        c.Gz = Gz;
+        usq = collide_increment2(s, (float *)s.pop[par ^ 1], nfp, f, P, c, rho);
+        ux = c.ux;
+        uy = c.uy;
+        uz = c.uz;
+    } else {
+        uint16_t *__restrict__ dst = (uint16_t *)s.pop[par ^ 1];
+        const CollK k = make_collk(s);
+        const Moments2 m = moments2<T>(P);
+        const Coll2 c = make_coll2(s, k, m, Gx, Gy, Gz, rho, usq);
+        const float sc = s.scale;
+        const float wsc0 = (float)d3q19_w(0) * sc, wsc1 = (float)d3q19_w(1) * sc, wsc2 = (float)d3q19_w(7) * sc;
+        uint32_t rng = mix32(f ^ step_seed);
+        rng = rng * 747796405u + 2891336453u;
+        const float2 o0 = fma2(v2(k.c1), unpack2<T>(P[0]), mul2(v2(wsc0), c.Kb));
+        __stcs((unsigned int *)(dst + f), Pack2<T>::rs(o0.x, o0.y, rng ^ (rng >> 15)));
+        {
+            const Cls2 w = make_cls2(c, k, wsc1);
+            collide2<T, 1>(dst, nfp, f, P[1], P[2], c, k, w, rng);
+            collide2<T, 3>(dst, nfp, f, P[3], P[4], c, k, w, rng);
+            collide2<T, 5>(dst, nfp, f, P[5], P[6], c, k, w, rng);
+        }
+        const Cls2 w = make_cls2(c, k, wsc2);
+        collide2<T, 7>(dst, nfp, f, P[7], P[8], c, k, w, rng);
+        collide2<T, 9>(dst, nfp, f, P[9], P[10], c, k, w, rng);
+        collide2<T, 11>(dst, nfp, f, P[11], P[12], c, k, w, rng);
+        collide2<T, 13>(dst, nfp, f, P[13], P[14], c, k, w, rng);
+        collide2<T, 15>(dst, nfp, f, P[15], P[16], c, k, w, rng);
+        collide2<T, 17>(dst, nfp, f, P[17], P[18], c, k, w, rng);
+        ux = c.ux;
+        uy = c.uy;
+        uz = c.uz;
+    }
+    if (cp.any) {
+        if (cp.act & 1u) s.ufield[f] = make_float4(ux.x, uy.x, uz.x, rho.x);
+        if (cp.act & 2u) s.ufield[f + 1] = make_float4(ux.y, uy.y, uz.y, rho.y);
+    }
+    if (!(usq.x < 0.09f) || !(usq.y < 0.09f)) atomicOr(s.status, ST_UNSTABLE);
 }
 
 template <typename T, bool EARLY>
 __device__ __forceinline__ void fluid_pair(const SimDev &s, int par, int fi, uint32_t step_seed) {
-    const uint16_t *__restrict__ src = (const uint16_t *)s.pop[par];
-    const uint32_t nfp = (uint32_t)s.nfp, f = (uint32_t)fi;
+    const T *__restrict__ src = (const T *)s.pop[par];
+    const size_t nfp = (size_t)s.nfp;
+    const uint32_t f = (uint32_t)fi;
     const uint32_t r = s.div_nx.div(f);
     const uint32_t x = f - r * (uint32_t)s.nx;
     const uint32_t z = s.div_nyf.div(r);
     const uint32_t y = r - z * (uint32_t)s.nyf;
-    const Nbr n = neighbours(s, (int)x, (int)y, (int)z);
-    const int dxm0 = n.dxm, dxp1 = ((int)x + 2 == s.nx) ? -(s.nx - 1) : 1;
+    const Rows n = source_rows(s, f, (int)y, (int)z);
+    const int xm = x == 0 ? s.nx - 1 : -1, xp = x + 2 == (uint32_t)s.nx ? 2 - s.nx : 2;
 
-    uint32_t P[NQ];
-#define LBIB_PULL2(q) P[q] = pull2<q>(src, nfp, f, n, dxm0, dxp1);
+    typename PairRaw<T>::type P[NQ];
+#define LBIB_PULL2(q) P[q] = pull2<T, q>(src, nfp, n, xm, xp);
     LBIB_PULL2(0) LBIB_PULL2(1) LBIB_PULL2(2) LBIB_PULL2(3) LBIB_PULL2(4) LBIB_PULL2(5) LBIB_PULL2(6)
     LBIB_PULL2(7) LBIB_PULL2(8) LBIB_PULL2(9) LBIB_PULL2(10) LBIB_PULL2(11) LBIB_PULL2(12) LBIB_PULL2(13)
     LBIB_PULL2(14) LBIB_PULL2(15) LBIB_PULL2(16) LBIB_PULL2(17) LBIB_PULL2(18)
@@ -780,7 +910,13 @@ __device__ __forceinline__ void fluid_pair(const SimDev &s, int par, int fi, uin
         dep_wait();
         dep_release();
     }
-    pair_update<T>(s, par, f, P, step_seed);
+    const uint32_t act = __ldcg(s.amask + (f >> 5));
+    const bool ylo = s.walls && y == 0, yhi = s.walls && y == (uint32_t)s.nyf - 1;
+    if (__any_sync(__activemask(), ylo || yhi)) {
+        if (ylo) bounce2<T, 1>(src, nfp, f, P);
+        if (yhi) bounce2<T, -1>(src, nfp, f, P);
+    }
+    pair_update<T>(s, par, f, P, step_seed, load_coupling(s, par, f, (act >> (f & 31)) & 3u));
 }
 
 // Pull offset of direction q in the fluid index space away from the
@@ -796,24 +932,21 @@ __host__ __device__ constexpr unsigned long long pack_e(int axis) {
 __device__ __forceinline__ int unpack_e(unsigned long long p, int q) { return (int)((p >> (2 * q)) & 3ull) - 1; }
 
 // The bulk L2 prefetch of the stretches of every plane that the CELLS cells
-// from fb on pull (thread q < 19 takes plane q).
+// from fb (>= 0) on pull (thread q < 19 takes plane q).
 template <int ESZ, int CELLS>
 __device__ __forceinline__ void prefetch_cells(const SimDev &s, const void *src, long long fb) {
     if (fb >= s.nf) return;
     const int q = (int)threadIdx.x;
     constexpr unsigned long long PX = pack_e(0), PY = pack_e(1), PZ = pack_e(2);
-    const long long off = -((long long)unpack_e(PX, q) + (long long)s.nx * unpack_e(PY, q) +
-                            (long long)s.nx * s.nyf * unpack_e(PZ, q));
-    long long a = fb + off - 16, b = fb + CELLS + off + 16;
-    if (a < 0) a = 0;
-    if (b > s.nfp) b = s.nfp;
+    const int off = unpack_e(PX, q) + s.nx * (unpack_e(PY, q) + s.nyf * unpack_e(PZ, q));
+    // 16 cells more on each side, clipped to the plane: 16-byte aligned start
+    // and size (nfp is a multiple of 64 and below 2^28)
+    constexpr int ALIGN = 16 / ESZ;
+    const int a = max((int)fb - off - 16, 0) & ~(ALIGN - 1);
+    const int b = min(((int)fb + CELLS - off + 16 + ALIGN - 1) & ~(ALIGN - 1), s.nfp);
     if (b <= a) return;
-    // 16-byte aligned start and size inside the plane (nfp is a multiple of 64)
-    const long long ab = (a * ESZ) & ~15ll;
-    long long bb = (b * ESZ + 15) & ~15ll;
-    if (bb > (long long)s.nfp * ESZ) bb = (long long)s.nfp * ESZ;
-    const char *p = (const char *)src + (long long)q * s.nfp * ESZ + ab;
-    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"((unsigned)(bb - ab)) : "memory");
+    const char *p = (const char *)src + ((size_t)(unsigned)q * (unsigned)s.nfp + (unsigned)a) * ESZ;
+    asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(p), "r"((unsigned)(b - a) * ESZ) : "memory");
 }
 
 // L2 prefetch for a later block: thread q < 19 of block b asks the L2 to

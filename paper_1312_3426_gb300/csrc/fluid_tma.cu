@@ -248,7 +248,10 @@ __global__ void __launch_bounds__(TMA_THREADS, 4) k_fluid_pair_tma(SimDev s, int
         asm volatile("fence.proxy.async.shared::cta;" ::: "memory");
         __syncwarp();
         if (lane == 0) mbar_arrive(empty + st);
-        if (mine) pair_update_act<T>(s, par, (uint32_t)(seg * tt.W + x + s.nx * row), P, seed, act);
+        if (mine) {
+            const uint32_t f = (uint32_t)(seg * tt.W + x + s.nx * row);
+            pair_update<T>(s, par, f, P, seed, load_coupling(s, par, f, act));
+        }
     }
 }
 

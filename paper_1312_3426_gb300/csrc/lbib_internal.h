@@ -254,6 +254,8 @@ cudaError_t launch_fluid(const SimDev &s, int par, long long t, cudaStream_t st,
 // the kernel launch_fluid picks (lbib_info out[7]): 0 one cell per thread,
 // 1 two cells per thread, 2 warp-specialised two cells per thread
 int fluid_kernel_kind(const SimDev &s);
+// L2 prefetch distance (in blocks) of a fluid launch of that kernel kind
+int fluid_prefetch(int prec, int kind, int sms);
 // fluid_tma.cu: the warp-specialised kernel and whether the shape allows it
 bool fluid_tma_shape(const SimDev &s);
 cudaError_t launch_fluid_tma(const SimDev &s, int par, uint32_t seed, cudaStream_t st);
