@@ -246,15 +246,23 @@ cudaError_t launch_repulsion(const SimDev &s, int max_nodes, cudaStream_t st) {
     return cudaGetLastError();
 }
 
-// Marks the cells around every node as active (after the mask was cleared).
+// Marks, after the mask was cleared, the corners of every node and those of
+// its position a step before (X - V): the force that step spread there is
+// still in the buffer that the coming fluid step clears at active cells.
+// With all 64 cells within one of a corner marked instead (which covered the
+// position before without reading V), 256x128x128 with 200 cells had 14.4%
+// of its cells active; the corners are 6.8%.
 __global__ void k_mark_all(SimDev s) {
     const int i = blockIdx.x * blockDim.x + threadIdx.x;
     if (i >= s.nn_total) return;
     const int NN = s.nn_total;
     const df x{s.Xh[i], s.Xl[i]}, y{s.Xh[NN + i], s.Xl[NN + i]}, z{s.Xh[2 * NN + i], s.Xl[2 * NN + i]};
     if (!isfinite(x.hi) || !isfinite(y.hi) || !isfinite(z.hi)) return;
-    const int3 c = lower_corner(x, y, z);
-    mark_halo(s, c.x, c.y, c.z);
+    mark_corners(s, x, y, z);
+    const df px = df_add(x, {-s.Vh[i], -s.Vl[i]}), py = df_add(y, {-s.Vh[NN + i], -s.Vl[NN + i]}),
+             pz = df_add(z, {-s.Vh[2 * NN + i], -s.Vl[2 * NN + i]});
+    const int3 c = lower_corner(x, y, z), p = lower_corner(px, py, pz);
+    if (p.x != c.x || p.y != c.y || p.z != c.z) mark_corners(s, px, py, pz);
 }
 
 cudaError_t launch_mark_all(const SimDev &s, cudaStream_t st) {

@@ -8,13 +8,14 @@
 //                    (plane stride nfp = nf rounded up to 64 elements), the
 //                    deviation h_i = f_i - w_i rho0 (times 2^s for FP16/BF16).
 //                    Step t pulls from pop[t&1] and writes pop[(t+1)&1].
-//   active cells     bit f of amask[nwords] marks the cells near objects: the
-//                    4x4x4 lattice nodes around every node (its 8
-//                    interpolation corners and a one-cell halo).  A node
-//                    marks them when its lower corner changes; marks persist
-//                    until a periodic reset, after which all nodes re-mark.
-//                    Nodes move less than one cell per step, so a node's
-//                    corners at the next step are always active already.
+//   active cells     bit f of amask[nwords] marks the cells the objects
+//                    touch: the 8 interpolation corners of every node, where
+//                    it stands and where it will stand at the next step (the
+//                    node update marks them, when its lower corner changes,
+//                    before the fluid update of the same step).  Marks
+//                    persist until a periodic reset, after which all nodes
+//                    mark the corners of their position and of the one a
+//                    step before (whose force the coming step clears).
 //   coupling force   G[2][nf] float4, dense, non-zero only at active cells.
 //                    Step t spreads into G[t&1]; the fluid step t adds
 //                    G[t&1] at active cells and zeroes G[(t+1)&1] there (the
