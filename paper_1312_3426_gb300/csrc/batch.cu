@@ -479,7 +479,12 @@ extern "C" lbib_status lbib_batch_step(lbib_sim *const *sims, int n, int n_steps
     // membrane forces of the current positions where they are not ready
     bool need_membrane = false;
     for (int i = 0; i < n; ++i) need_membrane |= !sims[i]->objs.empty() && !sims[i]->fel_valid;
-    if (e == cudaSuccess && need_membrane && n_steps > 0) e = launch_membrane_batch(st);
+    if (e == cudaSuccess && need_membrane && n_steps > 0) {
+        // the launch waits for ev_nodes: recorded here, on what st has done
+        // so far (a record of the captured graph cannot be waited for)
+        e = cudaEventRecord(g_plan.ev_nodes, st);
+        if (e == cudaSuccess) e = launch_membrane_batch(st);
+    }
 
     int done = 0;
     while (e == cudaSuccess && done < n_steps) {
