@@ -404,18 +404,19 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * slower than value 1 on a GB300, kept for comparison; lbib_batch_step runs
  * value 1 instead), 3 one cell per thread; FP32 storage ignores it.
  * LBIB_TUNE_NODE_THREADS: nodes per block of the node-update kernel (32,
- * 64, 128 or 256, default 256; lbib_batch_step takes the first
- * simulation's).  LBIB_TUNE_MEMBRANE_GROUP: objects per block of the
+ * 64, 128 or 256; reads 256 until set, while the step uses 64;
+ * lbib_batch_step takes the first simulation's).  LBIB_TUNE_MEMBRANE_GROUP: objects per block of the
  * membrane-force kernel (1..15, default 1); above 1 each object gets
  * LBIB_TUNE_MEMBRANE_THREADS threads of a block of group x threads threads
  * (at most 1024) and the cluster knobs do not apply; the step takes as
  * many objects per block as fit (threads and shared memory for the largest
  * template), at most the knob's value.
- * lbib_batch_step takes the first simulation's; it runs the objects within
- * a factor 2 of the largest in one launch and the others beside it in a
- * second (each with shared-memory slices sized for its own largest
- * object), with as many objects per block as fit, and keeps one object per
- * cluster when a single size class does not fit more than one.  LBIB_TUNE_EARLY_LAUNCH: 1 lets each node-update and
+ * lbib_batch_step takes the first simulation's; with a group above 1, or while
+ * neither it nor the threads are set, it runs the objects within a factor 2 of
+ * the largest in one launch and the others beside it in a second (each with
+ * shared-memory slices sized for its own largest object), with as many objects
+ * per block as fit, and keeps one object per cluster when a single size class
+ * does not fit more than one.  LBIB_TUNE_EARLY_LAUNCH: 1 lets each node-update and
  * fluid kernel of lbib_step after the first start while the kernel before
  * it finishes (programmatic dependent launch: the early part reads only data
  * that kernel does not write, and waits for it before the rest), 0 (default)

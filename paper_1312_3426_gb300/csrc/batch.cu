@@ -134,6 +134,10 @@ struct BatchPlan {
     // within a factor 2 of the largest, and the rest, whose largest has
     // rest_nodes nodes and rest_edges edges (0: one class)
     int n_big = 0, rest_nodes = 0, rest_edges = 0;
+    // threads per object of the two classes where neither that nor the group
+    // was set (0: g_plan.mthreads)
+    int big_threads = 0, rest_threads = 0;
+    bool mauto = false;
     int pf_cell = 0, pf_pair[2] = {};  // (pairs: 16-bit, FP32) L2 prefetch distances of the fluid launches (work items)
     cudaStream_t aux = nullptr;   // membrane kernel
     cudaStream_t aux2 = nullptr;  // membrane kernel of the smaller size class
@@ -177,7 +181,7 @@ static int fluid_group(const lbib_sim *s) {
 
 static bool plan_matches(lbib_sim *const *sims, int n, int cluster) {
     if ((int)g_plan.sims.size() != n || g_plan.cluster != cluster || g_plan.device != sims[0]->device ||
-        g_plan.nthreads != sims[0]->node_threads)
+        g_plan.nthreads != node_chunk(sims[0]))
         return false;
     for (int i = 0; i < n; ++i)
         if (g_plan.sims[i] != sims[i] || g_plan.serial[i] != sims[i]->serial ||
@@ -189,7 +193,7 @@ static bool plan_matches(lbib_sim *const *sims, int n, int cluster) {
 
 static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStream_t st) {
     g_plan.release();
-    const int nthreads = sims[0]->node_threads;  // node chunk of the batch
+    const int nthreads = node_chunk(sims[0]);  // of the batch
     if (!g_plan.aux) {
         int lo = 0, hi = 0;
         cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
@@ -268,6 +272,10 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
         g_plan.rest_nodes = std::max(g_plan.rest_nodes, nodes_of(mb[k]));
         g_plan.rest_edges = std::max(g_plan.rest_edges, sims[mb[k].x]->topo[sims[mb[k].x]->objs[mb[k].y].tid].ne);
     }
+    double fluid_us = 0.0;
+    for (int i = 0; i < n; ++i) fluid_us += fluid_time_us(sims[i]->d.nf, sims[i]->d.prec);
+    g_plan.big_threads = membrane_threads(g_plan.n_big, max_edges, fluid_us);
+    g_plan.rest_threads = membrane_threads((int)mb.size() - g_plan.n_big, g_plan.rest_edges, fluid_us);
     return cudaSuccess;
 }
 
@@ -280,48 +288,58 @@ static cudaError_t launch_repulsion_batch(cudaStream_t st) {
     return cudaSuccess;
 }
 
-// Membrane items [first, first + n) with up to G per block, each with a
-// shared-memory slice of `per` bytes (G drops to what fits).
-static cudaError_t launch_membrane_groups(cudaStream_t st, int first, int n, size_t per, int G) {
-    while (G > 1 && (G * g_plan.mthreads > 1024 || per * G > IB_SMEM_MAX)) --G;
-    static SmemAttr gattr;
-    cudaError_t e = gattr.ensure((const void *)k_batch_membrane_groups, per * G, false);
+// shared-memory limits of k_batch_membrane<false>, <true> and the groups kernel
+static SmemAttr g_attr_one, g_attr_global, g_attr_groups;
+
+// Membrane items [first, first + n) with up to G per block of T threads each,
+// each with a shared-memory slice of `per` bytes (G drops to what fits).
+static cudaError_t launch_membrane_groups(cudaStream_t st, int first, int n, size_t per, int G, int T) {
+    while (G > 1 && (G * T > 1024 || per * G > IB_SMEM_MAX)) --G;
+    const SimDev *sims = g_plan.d_sims;
+    const int2 *items = g_plan.d_items + g_plan.n_fl + g_plan.n_nd + first;
+    const void *fn = G > 1 ? (const void *)k_batch_membrane_groups : (const void *)k_batch_membrane<false>;
+    cudaError_t e = (G > 1 ? g_attr_groups : g_attr_one).ensure(fn, per * G, G == 1);
     if (e != cudaSuccess) return e;
-    const int blocks = (n + G - 1) / G;
-    k_batch_membrane_groups<<<blocks, G * g_plan.mthreads, per * G, st>>>(
-        (const SimDev *)g_plan.d_sims, (const int2 *)(g_plan.d_items + g_plan.n_fl + g_plan.n_nd + first), n,
-        g_plan.mthreads, (int)(per / sizeof(float)));
+    if (G > 1)
+        k_batch_membrane_groups<<<(n + G - 1) / G, G * T, per * G, st>>>(sims, items, n, T, (int)(per / sizeof(float)));
+    else
+        k_batch_membrane<false><<<n, T, per, st>>>(sims, items);
     return cudaGetLastError();
 }
 
 // On `st` (which waits for the node update): the membrane forces, then the
-// repulsion.  With several objects per block, the objects within a factor 2
-// of the largest run in one launch (their slices sized for the largest) and
-// the others beside it on a second stream (slices sized for theirs), so a
-// level-2 object does not hold the shared memory of a level-4 one.
+// repulsion.  The objects within a factor 2 of the largest run in one launch
+// (their slices sized for the largest) and the others beside it on a second
+// stream (slices sized for theirs), so a level-2 object does not hold the
+// shared memory of a level-4 one, and each class has threads for its size
+// (a step of 64 channels with objects of levels 2 to 4 takes 328 us, of 6
+// larger ones 44.6; 390 and 87.5 with one launch of 192 threads per object).
+// One launch, one object per cluster, where the threads or the cluster size
+// were set without a group, or a block cannot hold an object.
 static cudaError_t launch_membrane_batch(cudaStream_t st) {
     if (g_plan.n_mb == 0) return cudaSuccess;
     const int G = g_plan.mgroup;
     const size_t per = ib_smem_bytes(g_plan.max_nodes, g_plan.max_edges);
-    if (G > 1 && g_plan.n_big < g_plan.n_mb && per <= IB_SMEM_MAX) {
+    const bool own = g_plan.mauto && g_plan.cluster == 1;
+    const int T1 = own ? g_plan.big_threads : g_plan.mthreads, T2 = own ? g_plan.rest_threads : g_plan.mthreads;
+    if ((G > 1 || own) && g_plan.n_big < g_plan.n_mb && per <= IB_SMEM_MAX) {
         cudaError_t e;
         if ((e = cudaStreamWaitEvent(g_plan.aux2, g_plan.ev_nodes, 0)) != cudaSuccess) return e;
         if ((e = launch_membrane_groups(g_plan.aux2, g_plan.n_big, g_plan.n_mb - g_plan.n_big,
-                                        ib_smem_bytes(g_plan.rest_nodes, g_plan.rest_edges), G)) != cudaSuccess)
+                                        ib_smem_bytes(g_plan.rest_nodes, g_plan.rest_edges), G, T2)) != cudaSuccess)
             return e;
         if ((e = cudaEventRecord(g_plan.ev_rest, g_plan.aux2)) != cudaSuccess) return e;
-        if ((e = launch_membrane_groups(st, 0, g_plan.n_big, per, G)) != cudaSuccess) return e;
+        if ((e = launch_membrane_groups(st, 0, g_plan.n_big, per, G, T1)) != cudaSuccess) return e;
         if ((e = cudaStreamWaitEvent(st, g_plan.ev_rest, 0)) != cudaSuccess) return e;
         return launch_repulsion_batch(st);
     }
-    if (G > 1 && G * g_plan.mthreads <= 1024 && per * G <= IB_SMEM_MAX) {
-        cudaError_t e = launch_membrane_groups(st, 0, g_plan.n_mb, per, G);
+    if ((G > 1 || own) && G * T1 <= 1024 && per * G <= IB_SMEM_MAX) {
+        cudaError_t e = launch_membrane_groups(st, 0, g_plan.n_mb, per, G, T1);
         return e == cudaSuccess ? launch_repulsion_batch(st) : e;
     }
     const bool global = membrane_in_global(g_plan.max_nodes, g_plan.max_edges, g_plan.cluster);
     const size_t smem = global ? ib_smem_bytes(g_plan.max_nodes, 0) : per;
-    static SmemAttr attr[2];
-    cudaError_t e = attr[global].ensure(
+    cudaError_t e = (global ? g_attr_global : g_attr_one).ensure(
         global ? (const void *)k_batch_membrane<true> : (const void *)k_batch_membrane<false>, smem, true);
     if (e != cudaSuccess) return e;
     cudaLaunchConfig_t cfg = {};
@@ -454,9 +472,11 @@ extern "C" lbib_status lbib_batch_step(lbib_sim *const *sims, int n, int n_steps
             if (r != LBIB_OK) return r;
         }
     if (!plan_matches(sims, n, cluster)) e = build_plan(sims, n, cluster, st);
-    if (g_plan.mthreads != sims[0]->membrane_threads || g_plan.mgroup != sims[0]->membrane_group) {
+    if (g_plan.mthreads != sims[0]->membrane_threads || g_plan.mgroup != sims[0]->membrane_group ||
+        g_plan.mauto != sims[0]->membrane_auto) {
         g_plan.mthreads = sims[0]->membrane_threads;  // captured in the graph
         g_plan.mgroup = sims[0]->membrane_group;
+        g_plan.mauto = sims[0]->membrane_auto;
         g_plan.release_graph();
     }
     // descriptors (node arrays may have been reallocated, tables uploaded)

@@ -890,7 +890,7 @@ lbib_status lbib_step(lbib_sim *s, int n) {
         // node kernel releases only after it) before it waits for the mask
         // and the coupling buffer.
         const bool early = s->early_launch && i > 0 && !s->prof_now;
-        if (objects) LBIB_CUDA(s, launch_nodes(s->d, par, s->node_threads, s->stream, early), "node update");
+        if (objects) LBIB_CUDA(s, launch_nodes(s->d, par, node_chunk(s), s->stream, early), "node update");
         if (objects && s->overlap) {
             LBIB_CUDA(s, cudaEventRecord(s->ev_nodes, s->stream), "event");
             LBIB_CUDA(s, cudaStreamWaitEvent(s->aux, s->ev_nodes, 0), "event");
@@ -1274,6 +1274,7 @@ lbib_status lbib_set_tuning(lbib_sim *s, int key, int value) {
         if (value != 32 && value != 64 && value != 128 && value != 256)
             return fail(s, LBIB_ERR_ARG, "node threads must be 32, 64, 128 or 256");
         s->node_threads = value;
+        s->node_auto = false;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_EARLY_LAUNCH) {
