@@ -29,8 +29,9 @@ namespace lbib {
 // EARLY: the instantiation for an early (programmatic dependent) launch
 template <typename T, bool BC, bool EARLY>
 __global__ void __launch_bounds__(FLUID_THREADS, 5) k_fluid(SimDev s, uint32_t seed, int pf) {
-    prefetch_sources<sizeof(T), FLUID_THREADS>(s, s.pop[0], pf);
-    fluid_block<T, BC, EARLY>(s, 0, blockIdx.x * FLUID_THREADS, seed);
+    const int block = sweep_block(pf);
+    prefetch_sources<sizeof(T), FLUID_THREADS>(s, s.pop[0], block, pf);
+    fluid_block<T, BC, EARLY>(s, 0, block * FLUID_THREADS, seed);
 }
 
 // Even nx, no obstacles, no inlet: two cells per thread.  Both cells share
@@ -43,8 +44,9 @@ __global__ void __launch_bounds__(FLUID_THREADS, 5) k_fluid(SimDev s, uint32_t s
 // 455 -> 431 at 512x256x256, 47.1 -> 38.4 M).
 template <typename T, bool EARLY>
 __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>()) k_fluid_pair(SimDev s, uint32_t seed, int pf) {
-    prefetch_sources<sizeof(T), 2 * PAIR_THREADS>(s, s.pop[0], pf);
-    const int f = 2 * (int)(blockIdx.x * PAIR_THREADS + threadIdx.x);
+    const int block = sweep_block(pf);
+    prefetch_sources<sizeof(T), 2 * PAIR_THREADS>(s, s.pop[0], block, pf);
+    const int f = 2 * (block * PAIR_THREADS + (int)threadIdx.x);
     if (f < s.nf) fluid_pair<T, EARLY>(s, 0, f, seed);
 }
 
@@ -95,12 +97,12 @@ static cudaError_t launch_fluid_t(const SimDev &s, int par, uint32_t seed, int b
     }
     if (fluid_kernel_kind(s) == 1) {
         const unsigned pblocks = (unsigned)((s.nf / 2 + PAIR_THREADS - 1) / PAIR_THREADS);
-        const int pf = fluid_prefetch(s.prec, 1, sms);
+        const int pf = (par ? -1 : 1) * fluid_prefetch(s.prec, 1, sms);
         if (pdl) return launch_dep(k_fluid_pair<T, true>, pblocks, PAIR_THREADS, st, true, d, seed, pf);
         return launch_dep(k_fluid_pair<T, false>, pblocks, PAIR_THREADS, st, false, d, seed, pf);
     }
     const unsigned b = (unsigned)blocks;
-    const int pf = fluid_prefetch(s.prec, 0, sms);
+    const int pf = (par ? -1 : 1) * fluid_prefetch(s.prec, 0, sms);
     if (s.solid || s.in_on) {
         if (pdl) return launch_dep(k_fluid<T, true, true>, b, FLUID_THREADS, st, true, d, seed, pf);
         return launch_dep(k_fluid<T, true, false>, b, FLUID_THREADS, st, false, d, seed, pf);
