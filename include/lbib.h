@@ -392,10 +392,10 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * (0, default: one cluster per object; a small grid leaves most SMs to the
  * fluid kernel running beside it).  LBIB_TUNE_MEMBRANE_THREADS: threads per
  * block of the membrane-force kernel (a multiple of 32 in [32, 256];
- * reads 192 until set: while neither it nor LBIB_TUNE_MEMBRANE_GROUP is set
- * and one block takes an object, the step picks 128 to 1024 by the number
- * and size of the objects and the length of the fluid update beside them;
- * fewer threads leave more of each SM to the fluid kernel).  LBIB_TUNE_FLUID_KERNEL (16-bit storage): 0
+ * default 192: with that, one object per block and cluster size 1 the step
+ * picks 128 to 1024 by the number and size of the objects and the length of
+ * the fluid update beside them; fewer threads leave more of each SM to the
+ * fluid kernel).  LBIB_TUNE_FLUID_KERNEL (16-bit storage): 0
  * (default) and 1 the two-cells-per-thread kernel (where nx is even and
  * there are no obstacles or inlet), 2 the warp-specialised two-cells kernel
  * (a producer warp streams the populations through shared memory with bulk
@@ -404,15 +404,15 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * slower than value 1 on a GB300, kept for comparison; lbib_batch_step runs
  * value 1 instead), 3 one cell per thread; FP32 storage ignores it.
  * LBIB_TUNE_NODE_THREADS: nodes per block of the node-update kernel (32,
- * 64, 128 or 256; reads 256 until set, while the step uses 64;
+ * 64, 128 or 256; with the default, 256, the step takes 64;
  * lbib_batch_step takes the first simulation's).  LBIB_TUNE_MEMBRANE_GROUP: objects per block of the
  * membrane-force kernel (1..15, default 1); above 1 each object gets
  * LBIB_TUNE_MEMBRANE_THREADS threads of a block of group x threads threads
  * (at most 1024) and the cluster knobs do not apply; the step takes as
  * many objects per block as fit (threads and shared memory for the largest
  * template), at most the knob's value.
- * lbib_batch_step takes the first simulation's; with a group above 1, or while
- * neither it nor the threads are set, it runs the objects within a factor 2 of
+ * lbib_batch_step takes the first simulation's; with a group above 1, or with
+ * it and the threads at their defaults, it runs the objects within a factor 2 of
  * the largest in one launch and the others beside it in a second (each with
  * shared-memory slices sized for its own largest object), with as many objects
  * per block as fit, and keeps one object per cluster when a single size class
@@ -421,6 +421,8 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * it finishes (programmatic dependent launch: the early part reads only data
  * that kernel does not write, and waits for it before the rest), 0 (default)
  * launches them one after the other; lbib_batch_step ignores it.
+ * With every knob at its default, a small simulation (see csrc/steps.cu) runs
+ * the steps of one lbib_step call in one launch.
  * Results do not depend on the knobs beyond the order of
  * floating-point atomics (the three 16-bit kernels give identical
  * populations).  LBIB_ERR_ARG for an unknown key or an out-of-range value. */

@@ -60,7 +60,7 @@ __global__ void __launch_bounds__(FLUID_THREADS, 5)
     const int2 it = items[blockIdx.x];  // (simulation, block of cells)
     const SimDev &s = sims[it.x];
     const long long t = t_base[it.x] + step_off;
-    fluid_block<T, BC, false>(s, (int)(t & 1), it.y * FLUID_THREADS, step_seed(t));
+    fluid_block<T, BC, MODE_PLAIN>(s, (int)(t & 1), it.y * FLUID_THREADS, step_seed(t));
 }
 
 // Even nx, plain boundaries: two cells per thread.
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>())
     const SimDev &s = sims[it.x];
     const long long t = t_base[it.x] + step_off;
     const int f = 2 * (it.y * PAIR_THREADS + (int)threadIdx.x);
-    if (f < s.nf) fluid_pair<T, false>(s, (int)(t & 1), f, step_seed(t));
+    if (f < s.nf) fluid_pair<T, MODE_PLAIN>(s, (int)(t & 1), f, step_seed(t));
 }
 
 // NT nodes per work item (the plan's node chunk); 64 registers, a full
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(NT, 1024 / NT)
     const int2 it = items[blockIdx.x];  // (simulation, first node)
     const SimDev &s = sims[it.x];
     const int i = it.y + (int)threadIdx.x;
-    if (i < s.nn_total) node_step<false>(s, i, (int)((t_base[it.x] + step_off) & 1));
+    if (i < s.nn_total) node_step<MODE_PLAIN>(s, i, (int)((t_base[it.x] + step_off) & 1));
 }
 
 template <bool EG>
@@ -134,8 +134,8 @@ struct BatchPlan {
     // within a factor 2 of the largest, and the rest, whose largest has
     // rest_nodes nodes and rest_edges edges (0: one class)
     int n_big = 0, rest_nodes = 0, rest_edges = 0;
-    // threads per object of the two classes where neither that nor the group
-    // was set (0: g_plan.mthreads)
+    // threads per object of the two classes where that and the group have
+    // their defaults
     int big_threads = 0, rest_threads = 0;
     bool mauto = false;
     int pf_cell = 0, pf_pair[2] = {};  // (pairs: 16-bit, FP32) L2 prefetch distances of the fluid launches (work items)
@@ -314,8 +314,8 @@ static cudaError_t launch_membrane_groups(cudaStream_t st, int first, int n, siz
 // shared memory of a level-4 one, and each class has threads for its size
 // (a step of 64 channels with objects of levels 2 to 4 takes 328 us, of 6
 // larger ones 44.6; 390 and 87.5 with one launch of 192 threads per object).
-// One launch, one object per cluster, where the threads or the cluster size
-// were set without a group, or a block cannot hold an object.
+// One launch, one object per cluster, where other threads or another cluster
+// size were set without a group, or a block cannot hold an object.
 static cudaError_t launch_membrane_batch(cudaStream_t st) {
     if (g_plan.n_mb == 0) return cudaSuccess;
     const int G = g_plan.mgroup;

@@ -45,7 +45,7 @@ bool fluid_layout(const lbib_fluid_params &p, FluidLayout &L) {
     for (int k = 0; k < 2; ++k) { L.off_G[k] = o; o = align_up(o + (size_t)L.nf * 16, 256); }
     L.off_amask = o; o = align_up(o + (size_t)L.nwords * 4, 256);
     L.off_ufield = o; o = align_up(o + (size_t)L.nf * 16, 256);
-    L.off_status = o; o = align_up(o + 4, 256);
+    L.off_status = o; o = align_up(o + 4, 256);  // the word; counters of steps.cu from byte 64 on
     L.off_dropped = o; o = align_up(o + 24, 256);
     L.total = o;
     return true;
@@ -849,6 +849,13 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
 //   aux:    wait ev_nodes, membrane(t+1) -> ev_membrane
 // and `stream` has caught up with `aux` when the call returns.  With overlap
 // off every step is membrane(t), nodes(t), fluid(t) on `stream`.
+// Whether lbib_step runs its steps in one launch (steps.cu): a small simulation
+// whose launch knobs have their defaults, while no step is sampled.
+static bool many_steps(const lbib_sim *s) {
+    return s->overlap && s->membrane_auto && s->cluster == 1 && s->membrane_clusters == 0 && !s->early_launch &&
+           s->node_auto && !s->prof_on && !s->many_refused && s->d.fkern != 2 && steps_fit(s->d, s->max_nodes, s->max_edges);
+}
+
 lbib_status lbib_step(lbib_sim *s, int n) {
     LBIB_GUARD(s);
     if (n < 0) return fail(s, LBIB_ERR_ARG, "negative step count");
@@ -860,6 +867,28 @@ lbib_status lbib_step(lbib_sim *s, int n) {
         r = launch_membrane_timed(s, s->stream);
         if (r != LBIB_OK) return r;
         s->fel_valid = true;
+    }
+    if (n > 1 && many_steps(s)) {
+        // runs of steps up to the next mask reset, one launch each
+        while (n > 0) {
+            if (s->since_mark >= ACTIVE_RESET_STEPS) LBIB_CUDA(s, sim_remark(s, s->stream), "active cells");
+            const int m = std::min(n, ACTIVE_RESET_STEPS - s->since_mark);
+            const cudaError_t e =
+                launch_steps(s->d, s->max_nodes, s->max_edges, (long long)s->t, m, s->d.status + 16, s->stream);
+            if (e == cudaErrorCooperativeLaunchTooLarge) {  // a partial GPU: separate launches
+                cudaGetLastError();
+                s->many_refused = true;
+                break;
+            }
+            LBIB_CUDA(s, e, "steps");
+            s->since_mark += m;
+            s->t += m;
+            s->gmode = (int)((s->t - 1) & 1);
+            n -= m;
+        }
+        s->side_ok = false;  // no event marks the last node update
+        if (s->nn_total > 0) s->dev_newer = true;
+        if (n == 0) return LBIB_OK;
     }
     for (int i = 0; i < n; ++i) {
         const int par = (int)(s->t & 1);
@@ -1251,7 +1280,7 @@ lbib_status lbib_set_tuning(lbib_sim *s, int key, int value) {
     if (key == LBIB_TUNE_MEMBRANE_THREADS) {
         if (value < 32 || value > IB_THREADS || value % 32) return fail(s, LBIB_ERR_ARG, "membrane threads must be a multiple of 32 in [32, 256]");
         s->membrane_threads = value;
-        s->membrane_auto = false;
+        s->membrane_auto = s->membrane_threads == 192 && s->membrane_group == 1;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_MEMBRANE_CLUSTERS) {
@@ -1267,14 +1296,14 @@ lbib_status lbib_set_tuning(lbib_sim *s, int key, int value) {
     if (key == LBIB_TUNE_MEMBRANE_GROUP) {
         if (value < 1 || value > 15) return fail(s, LBIB_ERR_ARG, "membrane group must be in [1, 15]");
         s->membrane_group = value;
-        s->membrane_auto = false;
+        s->membrane_auto = s->membrane_threads == 192 && s->membrane_group == 1;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_NODE_THREADS) {
         if (value != 32 && value != 64 && value != 128 && value != 256)
             return fail(s, LBIB_ERR_ARG, "node threads must be 32, 64, 128 or 256");
         s->node_threads = value;
-        s->node_auto = false;
+        s->node_auto = value == IB_THREADS_DEFAULT;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_EARLY_LAUNCH) {

@@ -31,7 +31,7 @@ template <typename T, bool BC, bool EARLY>
 __global__ void __launch_bounds__(FLUID_THREADS, 5) k_fluid(SimDev s, uint32_t seed, int pf) {
     const int block = sweep_block(pf);
     prefetch_sources<sizeof(T), FLUID_THREADS>(s, s.pop[0], block, pf);
-    fluid_block<T, BC, EARLY>(s, 0, block * FLUID_THREADS, seed);
+    fluid_block<T, BC, EARLY ? MODE_EARLY : MODE_PLAIN>(s, 0, block * FLUID_THREADS, seed);
 }
 
 // Even nx, no obstacles, no inlet: two cells per thread.  Both cells share
@@ -47,7 +47,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>()) k_fluid_pair(S
     const int block = sweep_block(pf);
     prefetch_sources<sizeof(T), 2 * PAIR_THREADS>(s, s.pop[0], block, pf);
     const int f = 2 * (block * PAIR_THREADS + (int)threadIdx.x);
-    if (f < s.nf) fluid_pair<T, EARLY>(s, 0, f, seed);
+    if (f < s.nf) fluid_pair<T, EARLY ? MODE_EARLY : MODE_PLAIN>(s, 0, f, seed);
 }
 
 static bool pair_shape(const SimDev &s) { return (s.nx & 1) == 0 && !s.solid && !s.in_on; }

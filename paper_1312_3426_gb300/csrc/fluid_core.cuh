@@ -95,6 +95,12 @@ struct Pack2<__nv_bfloat16> {
     }
 };
 
+template <int MODE, typename V>
+__device__ __forceinline__ V ld_pop(const V *p) {
+    if constexpr (MODE == MODE_MANY) return __ldcg(p);
+    else return __ldg(p);
+}
+
 // Raw storage access for the step kernel: the stored number as float (the
 // deviation times 2^s for FP16/BF16), and the store of two such numbers at
 // two addresses, rounded together with the random bits r.
@@ -102,7 +108,8 @@ template <typename T>
 struct Raw;
 template <>
 struct Raw<float> {
-    static __device__ __forceinline__ float ld(const float *p) { return __ldg(p); }
+    template <int MODE>
+    static __device__ __forceinline__ float ld(const float *p) { return ld_pop<MODE>(p); }
     static __device__ __forceinline__ void st2(float *p, float *q, float a, float b, uint32_t) {
         __stcs(p, a);
         __stcs(q, b);
@@ -110,7 +117,10 @@ struct Raw<float> {
 };
 template <>
 struct Raw<__half> {
-    static __device__ __forceinline__ float ld(const __half *p) { return __half2float(__ldg(p)); }
+    template <int MODE>
+    static __device__ __forceinline__ float ld(const __half *p) {
+        return __half2float(__ushort_as_half(ld_pop<MODE>((const unsigned short *)p)));
+    }
     static __device__ __forceinline__ void st2(__half *p, __half *q, float a, float b, uint32_t r) {
         const uint32_t d = Pack2<__half>::rs(a, b, r);
         __stcs((unsigned short *)p, (unsigned short)d);
@@ -119,8 +129,9 @@ struct Raw<__half> {
 };
 template <>
 struct Raw<__nv_bfloat16> {
+    template <int MODE>
     static __device__ __forceinline__ float ld(const __nv_bfloat16 *p) {
-        return __uint_as_float((uint32_t)__ldg((const unsigned short *)p) << 16);
+        return __uint_as_float((uint32_t)ld_pop<MODE>((const unsigned short *)p) << 16);
     }
     static __device__ __forceinline__ void st2(__nv_bfloat16 *p, __nv_bfloat16 *q, float a, float b, uint32_t r) {
         const uint32_t d = Pack2<__nv_bfloat16>::rs(a, b, r);
@@ -133,7 +144,7 @@ struct Raw<__nv_bfloat16> {
 // to x - 1 and x + 1, periodic; walls not considered).  In the
 // boundary-condition variant (BC) a population coming from an obstacle cell
 // is the cell's own opposite one, as at the walls.
-template <typename T, int Q, bool BC>
+template <typename T, int Q, bool BC, int MODE>
 __device__ __forceinline__ float pull(const SimDev &s, const T *__restrict__ src, size_t nfp, const Rows &n, int xm,
                                       int xp) {
     constexpr int ex = d3q19_ex(Q), ey = d3q19_ey(Q), ez = d3q19_ez(Q);
@@ -141,19 +152,19 @@ __device__ __forceinline__ float pull(const SimDev &s, const T *__restrict__ src
     if constexpr (ex == 1) g += (uint32_t)xm;
     if constexpr (ex == -1) g += (uint32_t)xp;
     if (BC && Q != 0 && s.solid && solid_bit(s, (int)g))
-        return Raw<T>::ld(src + (size_t)d3q19_opp(Q) * nfp + n.row[1][1]);
-    return Raw<T>::ld(src + (size_t)Q * nfp + g);
+        return Raw<T>::template ld<MODE>(src + (size_t)d3q19_opp(Q) * nfp + n.row[1][1]);
+    return Raw<T>::template ld<MODE>(src + (size_t)Q * nfp + g);
 }
 
 // Bounce-back at a wall row (the row below, EY = 1, or above, EY = -1, is
 // solid): the populations with that ey are the cell's own opposite ones.
 // Their periodic pulls, already on the way, are replaced; only warps with a
 // cell of a wall row come here.
-template <typename T, int EY>
+template <typename T, int EY, int MODE>
 __device__ __forceinline__ void bounce(const T *__restrict__ src, size_t nfp, uint32_t f, float (&h)[NQ]) {
 #pragma unroll
     for (int q = 1; q < NQ; ++q)
-        if (d3q19_ey(q) == EY) h[q] = Raw<T>::ld(src + (size_t)d3q19_opp(q) * nfp + f);
+        if (d3q19_ey(q) == EY) h[q] = Raw<T>::template ld<MODE>(src + (size_t)d3q19_opp(q) * nfp + f);
 }
 
 // BGK + Guo update of the opposite pair (Q, Q+1) (e_{Q+1} = -e_Q, same
@@ -393,8 +404,9 @@ __device__ __forceinline__ float collide_increment(const SimDev &s, float *__res
     c.ux = ux;
     c.uy = uy;
     c.uz = uz;
-    const float usq = ux * ux + uy * uy + uz * uz;
-    c.m3uG = -3.0f * (ux * Gx + uy * Gy + uz * Gz);
+    // explicit order: the two-cells kernel's packed instructions, bit for bit
+    const float usq = __fmaf_rn(uz, uz, __fmaf_rn(uy, uy, __fmul_rn(ux, ux)));
+    c.m3uG = __fmul_rn(-3.0f, __fmaf_rn(uz, Gz, __fmaf_rn(uy, Gy, __fmul_rn(ux, Gx))));
     c.K = fmaf(-1.5f * rho, usq, drho);
     c.r45 = 4.5f * rho;
     constexpr float w0 = (float)(1.0 / 3.0);
@@ -422,10 +434,10 @@ __device__ __forceinline__ uint32_t active_word(const SimDev &s, int f) {
     return (w < s.nwords) ? __ldcg(s.amask + w) : 0u;
 }
 
-// EARLY: the kernel may be launched early (programmatic dependent launch):
+// MODE_EARLY (the kernel may be launched early, programmatic dependent launch):
 // the mask word is read after dep_wait(); otherwise it is `act`, read by the
 // caller before the pulls.
-template <typename T, bool BC, bool EARLY>
+template <typename T, bool BC, int MODE>
 __device__ __forceinline__ void fluid_cell(const SimDev &s, int par, int fi, uint32_t act, uint32_t step_seed) {
     static_assert(d3q19_opp(1) == 2 && d3q19_opp(17) == 18, "directions 2k-1, 2k must be opposite");
     const T *__restrict__ src = (const T *)s.pop[par];
@@ -440,21 +452,21 @@ __device__ __forceinline__ void fluid_cell(const SimDev &s, int par, int fi, uin
     const int xm = x == 0 ? s.nx - 1 : -1, xp = x == (uint32_t)s.nx - 1 ? 1 - s.nx : 1;
 
     float h[NQ];
-#define LBIB_PULL(q) h[q] = pull<T, q, BC>(s, src, nfp, n, xm, xp);
+#define LBIB_PULL(q) h[q] = pull<T, q, BC, MODE>(s, src, nfp, n, xm, xp);
     LBIB_PULL(0) LBIB_PULL(1) LBIB_PULL(2) LBIB_PULL(3) LBIB_PULL(4) LBIB_PULL(5) LBIB_PULL(6)
     LBIB_PULL(7) LBIB_PULL(8) LBIB_PULL(9) LBIB_PULL(10) LBIB_PULL(11) LBIB_PULL(12) LBIB_PULL(13)
     LBIB_PULL(14) LBIB_PULL(15) LBIB_PULL(16) LBIB_PULL(17) LBIB_PULL(18)
 #undef LBIB_PULL
     const bool ylo = s.walls && y == 0, yhi = s.walls && y == (uint32_t)s.nyf - 1;
     if (__any_sync(__activemask(), ylo || yhi)) {
-        if (ylo) bounce<T, 1>(src, nfp, f, h);
-        if (yhi) bounce<T, -1>(src, nfp, f, h);
+        if (ylo) bounce<T, 1, MODE>(src, nfp, f, h);
+        if (yhi) bounce<T, -1, MODE>(src, nfp, f, h);
     }
 
     if (BC && s.in_on) inlet_cell(s, (int)x, (int)y + s.walls, (int)z, h);
     // the populations pulled above were written by the previous fluid step;
     // the mask and the coupling buffer below by the node update of this one
-    if constexpr (EARLY) {
+    if constexpr (MODE == MODE_EARLY) {
         dep_wait();
         dep_release();
         act = active_word(s, fi);
@@ -557,19 +569,26 @@ constexpr int pair_blocks() {  // per SM, at 96 (FP32) and 80 registers a thread
 template <typename T>
 struct PairRaw {
     using type = uint32_t;
+    template <int MODE>
     static __device__ __forceinline__ uint32_t ld(const T *p, uint32_t i) {
-        return __ldg((const unsigned int *)(p + i));
+        return ld_pop<MODE>((const unsigned int *)(p + i));
     }
+    template <int MODE>
     static __device__ __forceinline__ uint32_t ld(const T *p, uint32_t i, uint32_t j) {
-        return (uint32_t)__ldg((const unsigned short *)p + i) | ((uint32_t)__ldg((const unsigned short *)p + j) << 16);
+        return (uint32_t)ld_pop<MODE>((const unsigned short *)p + i) |
+               ((uint32_t)ld_pop<MODE>((const unsigned short *)p + j) << 16);
     }
 };
 template <>
 struct PairRaw<float> {
     using type = float2;
-    static __device__ __forceinline__ float2 ld(const float *p, uint32_t i) { return __ldg((const float2 *)(p + i)); }
+    template <int MODE>
+    static __device__ __forceinline__ float2 ld(const float *p, uint32_t i) {
+        return ld_pop<MODE>((const float2 *)(p + i));
+    }
+    template <int MODE>
     static __device__ __forceinline__ float2 ld(const float *p, uint32_t i, uint32_t j) {
-        return make_float2(__ldg(p + i), __ldg(p + j));
+        return make_float2(ld_pop<MODE>(p + i), ld_pop<MODE>(p + j));
     }
 };
 
@@ -580,24 +599,24 @@ struct PairRaw<float> {
 // slowed the kernel 6% at 512x256x256, where the x-shifted lines shared by
 // neighbouring warps were evicted in between; the loads keep the default
 // policy.
-template <typename T, int Q>
+template <typename T, int Q, int MODE>
 __device__ __forceinline__ typename PairRaw<T>::type pull2(const T *__restrict__ src, size_t nfp, const Rows &n, int xm,
                                                            int xp) {
     constexpr int ex = d3q19_ex(Q), ey = d3q19_ey(Q), ez = d3q19_ez(Q);
     const T *p = src + (size_t)Q * nfp;
     const uint32_t o = n.row[1 + ey][1 + ez];
-    if constexpr (ex == 0) return PairRaw<T>::ld(p, o);
-    else if constexpr (ex == 1) return PairRaw<T>::ld(p, o + (uint32_t)xm, o);  // from x - 1 and x
-    else return PairRaw<T>::ld(p, o + 1u, o + (uint32_t)xp);                    // from x + 1 and x + 2
+    if constexpr (ex == 0) return PairRaw<T>::template ld<MODE>(p, o);
+    else if constexpr (ex == 1) return PairRaw<T>::template ld<MODE>(p, o + (uint32_t)xm, o);  // from x - 1 and x
+    else return PairRaw<T>::template ld<MODE>(p, o + 1u, o + (uint32_t)xp);                    // from x + 1 and x + 2
 }
 
 // bounce() of the pair
-template <typename T, int EY>
+template <typename T, int EY, int MODE>
 __device__ __forceinline__ void bounce2(const T *__restrict__ src, size_t nfp, uint32_t f,
                                         typename PairRaw<T>::type (&P)[NQ]) {
 #pragma unroll
     for (int q = 1; q < NQ; ++q)
-        if (d3q19_ey(q) == EY) P[q] = PairRaw<T>::ld(src + (size_t)d3q19_opp(q) * nfp, f);
+        if (d3q19_ey(q) == EY) P[q] = PairRaw<T>::template ld<MODE>(src + (size_t)d3q19_opp(q) * nfp, f);
 }
 
 // The arithmetic of the two cells runs in packed FP32 instructions (sm_100
@@ -888,7 +907,7 @@ __device__ __forceinline__ void pair_update(const SimDev &s, int par, uint32_t f
     if (!(usq.x < 0.09f) || !(usq.y < 0.09f)) atomicOr(s.status, ST_UNSTABLE);
 }
 
-template <typename T, bool EARLY>
+template <typename T, int MODE>
 __device__ __forceinline__ void fluid_pair(const SimDev &s, int par, int fi, uint32_t step_seed) {
     const T *__restrict__ src = (const T *)s.pop[par];
     const size_t nfp = (size_t)s.nfp;
@@ -901,20 +920,20 @@ __device__ __forceinline__ void fluid_pair(const SimDev &s, int par, int fi, uin
     const int xm = x == 0 ? s.nx - 1 : -1, xp = x + 2 == (uint32_t)s.nx ? 2 - s.nx : 2;
 
     typename PairRaw<T>::type P[NQ];
-#define LBIB_PULL2(q) P[q] = pull2<T, q>(src, nfp, n, xm, xp);
+#define LBIB_PULL2(q) P[q] = pull2<T, q, MODE>(src, nfp, n, xm, xp);
     LBIB_PULL2(0) LBIB_PULL2(1) LBIB_PULL2(2) LBIB_PULL2(3) LBIB_PULL2(4) LBIB_PULL2(5) LBIB_PULL2(6)
     LBIB_PULL2(7) LBIB_PULL2(8) LBIB_PULL2(9) LBIB_PULL2(10) LBIB_PULL2(11) LBIB_PULL2(12) LBIB_PULL2(13)
     LBIB_PULL2(14) LBIB_PULL2(15) LBIB_PULL2(16) LBIB_PULL2(17) LBIB_PULL2(18)
 #undef LBIB_PULL2
-    if constexpr (EARLY) {  // as in fluid_cell
+    if constexpr (MODE == MODE_EARLY) {  // as in fluid_cell
         dep_wait();
         dep_release();
     }
     const uint32_t act = __ldcg(s.amask + (f >> 5));
     const bool ylo = s.walls && y == 0, yhi = s.walls && y == (uint32_t)s.nyf - 1;
     if (__any_sync(__activemask(), ylo || yhi)) {
-        if (ylo) bounce2<T, 1>(src, nfp, f, P);
-        if (yhi) bounce2<T, -1>(src, nfp, f, P);
+        if (ylo) bounce2<T, 1, MODE>(src, nfp, f, P);
+        if (yhi) bounce2<T, -1, MODE>(src, nfp, f, P);
     }
     pair_update<T>(s, par, f, P, step_seed, load_coupling(s, par, f, (act >> (f & 31)) & 3u));
 }
@@ -984,12 +1003,12 @@ __host__ __device__ __forceinline__ uint32_t step_seed(long long t) {
 }
 
 
-// One block of FLUID_THREADS consecutive fluid cells starting at f0.
-template <typename T, bool BC, bool EARLY>
+// One block of consecutive fluid cells starting at f0 (a multiple of 32).
+template <typename T, bool BC, int MODE>
 __device__ __forceinline__ void fluid_block(const SimDev &s, int par, int f0, uint32_t step_seed) {
     const int f = f0 + (int)threadIdx.x;
-    const uint32_t act = EARLY ? 0u : active_word(s, f);
-    if (f < s.nf) fluid_cell<T, BC, EARLY>(s, par, f, act, step_seed);
+    const uint32_t act = MODE == MODE_EARLY ? 0u : active_word(s, f);
+    if (f < s.nf) fluid_cell<T, BC, MODE>(s, par, f, act, step_seed);
 }
 
 }  // namespace lbib

@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(1024, 1) k_membrane_groups(SimDev s, int T, in
 template <int NT, bool EARLY>
 __global__ void __launch_bounds__(NT, 1024 / NT) k_nodes(SimDev s, int par) {
     const int i = blockIdx.x * NT + threadIdx.x;
-    if (i < s.nn_total) node_step<EARLY>(s, i, par);
+    if (i < s.nn_total) node_step<EARLY ? MODE_EARLY : MODE_PLAIN>(s, i, par);
 }
 
 bool membrane_in_global(int max_nodes, int max_edges, int cluster) {

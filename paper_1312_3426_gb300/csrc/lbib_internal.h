@@ -217,6 +217,12 @@ struct SmemAttr {
     }
 };
 
+// How the body of a step runs: by a kernel of its own; by one that may be
+// launched early (programmatic dependent launch); or as one of many steps of
+// one launch, where populations and velocity samples were written by other
+// blocks of the same kernel and have to be read through the L2.
+enum : int { MODE_PLAIN = 0, MODE_EARLY = 1, MODE_MANY = 2 };
+
 // ---- programmatic dependent launch -------------------------------------------
 // A kernel launched with `pdl` may start while the kernel before it in the
 // stream finishes.  It reads, before dep_wait(), only data that no kernel
@@ -275,6 +281,14 @@ constexpr int MASS_SCRATCH_SLOTS = 1024;
 constexpr int MASS_SCRATCH_DEVICES = 64;
 cudaError_t mass_scratch(double **ptr);
 cudaError_t launch_mass_partials(const SimDev &s, int pop_par, double *part, int blocks, cudaStream_t st);
+
+// ---- steps.cu ------------------------------------------------------------
+// n steps from step t on in one cooperative launch, where steps_fit; sync:
+// 192 device bytes of counters.  The membrane forces of the first step's
+// positions are in Fel, and those of the final positions will be.
+bool steps_fit(const SimDev &s, int max_nodes, int max_edges);
+cudaError_t launch_steps(const SimDev &s, int max_nodes, int max_edges, long long t, int n, unsigned *sync,
+                         cudaStream_t st);
 
 // ---- launchers (ib.cu) -----------------------------------------------------
 // membrane part: clusters of `cluster` blocks, one per object or at most

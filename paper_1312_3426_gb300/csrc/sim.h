@@ -78,11 +78,11 @@ struct lbib_sim {
     bool overlap = true;                // membrane of step t+1 on `aux` during fluid of step t
     int membrane_clusters = 0;          // clusters of the membrane kernel (0: one per object)
     int membrane_threads = 192;         // block size of the membrane kernel (per object) ...
-    bool membrane_auto = true;          // ... unless neither it nor the group was set: membrane_threads()
+    bool membrane_auto = true;          // ... unless it and the group have their defaults: membrane_threads()
     int membrane_group = 1;             // objects per block of the membrane kernel
     bool early_launch = false;          // programmatic dependent launch of the node and fluid kernels
     int node_threads = lbib::IB_THREADS_DEFAULT;  // nodes per block of the node kernel ...
-    bool node_auto = true;                        // ... unless not set: node_chunk()
+    bool node_auto = true;                        // ... unless it has its default: node_chunk()
 
     double rep_obj[3] = {0, 1, 0};      // soft-sphere repulsion (a, n, cutoff) between objects
     double rep_wall[3] = {0, 1, 0};     // and against the walls
@@ -91,6 +91,7 @@ struct lbib_sim {
     int rep_cap_obj = 0;                // objects the buffers hold
     size_t rep_bytes = 0;
 
+    bool many_refused = false;   // the device did not hold the blocks of a many-steps launch (steps.cu)
     bool prof_on = false;        // per-phase CUDA-event timing
     int prof_every = 1;          // ... of every prof_every-th step
     bool prof_now = false;       // the step being enqueued is timed
@@ -113,7 +114,7 @@ lbib_status sim_upload(lbib_sim *s);
 lbib_status sim_prepare_step(lbib_sim *s);
 lbib_status sim_edge_scratch(lbib_sim *s);
 cudaError_t sim_remark(lbib_sim *s, cudaStream_t st);
-// Nodes per block of the node kernel: 64 unless set.  A node waits for two
+// Nodes per block of the node kernel: 64 while the knob has its default.  A node waits for two
 // rounds of memory, one after the other, and small blocks leave and refill an
 // SM one by one (steps with 64 against 256: 3 cells 64x48x48 21.8 / 22.6 us,
 // 20 cells 117x70x66 26.4 / 27.3, 200 cells 256x128x128 FP32 126.9 / 128.1,

@@ -1,0 +1,184 @@
+// Many steps of one small simulation in one launch.
+//
+// A step of a small channel is a chain of short kernels (node update, then
+// membrane forces of the next step beside the fluid update), and the launches
+// and cross-stream events between them take longer than the kernels: 14.5 us
+// a step for one sphere in a 40x20x20 channel, 7 of them between kernels, and
+// the host enqueues no faster than 11 us a step.  Here one cooperative launch
+// runs all steps of a call, with two barriers over its blocks in each:
+//   node update    32 nodes per warp, spread over all blocks (on one SM the
+//                  scattered gathers and reductions of a level-3 cell's 642
+//                  nodes take 7 us, at about one sector a cycle);
+//   [barrier]
+//   then, by role  the first blocks: the membrane forces of one object each, for
+//                  the next step; the others: the fluid cells, in tiles;
+//   [barrier]
+// The barriers are counters in global memory that only grow (reset before the
+// launch), added to after a block barrier and a fence, read with acquire by
+// one thread before a block barrier.  All blocks are resident (cooperative
+// launch) and arrive at every barrier in order, so every wait ends; as
+// everywhere it is bounded by the global timer all the same: one that runs out
+// sets ST_TIMEOUT and the block leaves.  What another block writes during the
+// launch is read through the L2 (populations, velocity samples, mask, forces,
+// and the positions of an object by its membrane block); a node's own state
+// stays with its thread.
+#include "fluid_core.cuh"
+#include "ib_core.cuh"
+
+namespace lbib {
+
+// One block per SM.  768 threads (80 registers each) take a level-3 cell's 642
+// nodes in one round; the FP32 two-cells update spills at 80 registers, so
+// its blocks have 512 (128x64x64 without objects 12.0 us a step against 18.7).
+template <typename T, bool PAIR>
+constexpr int STEPS_THREADS = sizeof(T) == 4 && PAIR ? 512 : 768;
+constexpr unsigned long long STEPS_WAIT_NS = 10000000000ull;
+
+extern __shared__ float steps_smem[];
+
+__device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
+    unsigned v;
+    asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+    return v;
+}
+
+// Until *c has reached target (all threads of the block call it); false when
+// the bound ran out.
+__device__ __forceinline__ bool steps_wait(const SimDev &s, const unsigned *c, unsigned target) {
+    bool late = false;
+    if (threadIdx.x == 0 && ld_acquire(c) < target) {
+        unsigned long long t0, t1;
+        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+        for (unsigned i = 1; ld_acquire(c) < target; ++i) {
+            if ((i & 1023u) != 0u) continue;
+            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
+            if (t1 - t0 > STEPS_WAIT_NS) {
+                atomicOr(s.status, ST_TIMEOUT);
+                late = true;
+                break;
+            }
+        }
+    }
+    return __syncthreads_or(late) == 0;
+}
+
+__device__ __forceinline__ void steps_signal(unsigned *c) {
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        __threadfence();
+        atomicAdd(c, 1u);
+    }
+}
+
+// PAIR: two cells per thread (else one; BC: obstacles or an inlet)
+template <typename T, bool PAIR, bool BC>
+__global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, long long t0, int n, unsigned *sync) {
+    constexpr int THREADS = STEPS_THREADS<T, PAIR>, CELLS = PAIR ? 2 * THREADS : THREADS;
+    unsigned *nodes_done = sync, *done = sync + 32;
+    const unsigned blocks = gridDim.x;
+    const int nobj = s.nobj, b = (int)blockIdx.x, nfluid = (int)blocks - nobj;
+    const int tiles = (s.nf + CELLS - 1) / CELLS;
+    for (int k = 0; k < n; ++k) {
+        const long long t = t0 + k;
+        const int par = (int)(t & 1);
+        if (k > 0 && !steps_wait(s, done, blocks * (unsigned)k)) return;
+        if (nobj > 0) {
+            for (int i = 32 * (int)((threadIdx.x >> 5) * blocks + blockIdx.x); i < s.nn_total; i += THREADS * (int)blocks)
+                if (i + (int)(threadIdx.x & 31) < s.nn_total) node_step<MODE_MANY>(s, i + (int)(threadIdx.x & 31), par);
+            steps_signal(nodes_done);
+            if (!steps_wait(s, nodes_done, blocks * (unsigned)(k + 1))) return;
+        }
+        if (b < nobj) {
+            membrane_object<false, MODE_MANY>(s, b, steps_smem, BlockTeam());
+        } else {
+            const uint32_t seed = step_seed(t);
+            for (int tile = b - nobj; tile < tiles; tile += nfluid) {
+                const int f0 = tile * CELLS;
+                if constexpr (PAIR) {
+                    const int f = f0 + 2 * (int)threadIdx.x;
+                    if (f < s.nf) fluid_pair<T, MODE_MANY>(s, par, f, seed);
+                } else {
+                    fluid_block<T, BC, MODE_MANY>(s, par, f0, seed);
+                }
+            }
+        }
+        steps_signal(done);
+    }
+}
+
+// Two cells per thread where the shape allows; FP32 (the same bits either
+// way) only where one cell per thread takes more than two rounds of the
+// blocks (64x48x48 with 3 cells 12.7 against 14.6 us a step).
+static bool steps_pair(const SimDev &s) {
+    if (fluid_kernel_kind(s) == 0) return false;
+    return s.prec != LBIB_POP_F32 || s.nf > 2 * STEPS_THREADS<float, false> * (device_sms() - s.nobj);
+}
+static int steps_tiles(const SimDev &s) {
+    const int cells = !steps_pair(s)             ? STEPS_THREADS<float, false>
+                      : s.prec == LBIB_POP_F32 ? 2 * STEPS_THREADS<float, true>
+                                               : 2 * STEPS_THREADS<__half, true>;
+    return (s.nf + cells - 1) / cells;
+}
+
+// Blocks for the fluid cells: what is left of the SMs, one tile each if that is
+// fewer.  Beside objects, whose membrane blocks take as long as two or three
+// rounds of tiles, half as many do (64x48x48 with 3 cells: 49 blocks instead of
+// 95 at 12.9 us a step), and simulations on other streams find room (8 of
+// these on 8 streams 4.5 us a simulation and step against 12.8 with 95 blocks,
+// 7.9 with separate launches, which the host bounds).
+static int steps_fluid_blocks(const SimDev &s) {
+    const int sms = device_sms() - s.nobj, tiles = steps_tiles(s);
+    if (s.nobj > 0 && tiles > sms / 4 && tiles <= sms) return (tiles + 1) / 2;
+    return tiles < sms ? tiles : sms;
+}
+
+// Up to 8 rounds of the fluid blocks (without objects 32 tiles to 5 rounds),
+// and objects on half of the SMs at most.  us a step, one launch against
+// separate ones:
+//   sphere 40x20x20                 9.4 / 15.0
+//   no objects 101x37x53            6.4 /  8.3    128x96x96 FP16  16.5 / 18.5
+//   3 cells 64x48x48 FP16          12.9 / 22.4
+//   20 cells 117x70x66 FP32        20.3 / 25.6
+//   20 cells 128x64x64 FP32        17.2 / 24.3    FP16  15.2 / 24.2
+//   8 level-4 cells 128x64x64 FP32 30.7 / 39.3
+//   20 cells 96x96x96 FP32         31.0 / 32.9    160x96x96 FP16  32.6 / 34.3
+// beyond (10 rounds at 160x96x96 FP32, 160x128x96 FP16) they are equal.
+bool steps_fit(const SimDev &s, int max_nodes, int max_edges) {
+    const int sms = device_sms();
+    if (s.rep_on || (s.nobj > 0 && ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX)) return false;
+    const int tiles = steps_tiles(s);
+    if (s.nobj == 0) return tiles >= 32 && tiles <= 5 * sms;
+    return 2 * s.nobj <= sms && tiles <= 8 * (sms - s.nobj);
+}
+
+template <typename T, bool PAIR, bool BC>
+static cudaError_t launch_steps_t(const SimDev &s, size_t smem, long long t, int n, unsigned *sync, cudaStream_t st) {
+    static SmemAttr attr;
+    void *fn = (void *)k_steps<T, PAIR, BC>;
+    cudaError_t e = attr.ensure(fn, smem, false);
+    if (e == cudaSuccess) e = cudaMemsetAsync(sync, 0, 192, st);
+    if (e != cudaSuccess) return e;
+    const int fluid = steps_fluid_blocks(s);
+    SimDev d = s;
+    void *args[] = {&d, &t, &n, &sync};
+    return cudaLaunchCooperativeKernel(fn, dim3((unsigned)(s.nobj + fluid)), dim3(STEPS_THREADS<T, PAIR>), args, smem, st);
+}
+
+template <typename T>
+static cudaError_t launch_steps_v(const SimDev &s, size_t smem, long long t, int n, unsigned *sync, cudaStream_t st) {
+    if (steps_pair(s)) return launch_steps_t<T, true, false>(s, smem, t, n, sync, st);
+    if (s.solid || s.in_on) return launch_steps_t<T, false, true>(s, smem, t, n, sync, st);
+    return launch_steps_t<T, false, false>(s, smem, t, n, sync, st);
+}
+
+cudaError_t launch_steps(const SimDev &s, int max_nodes, int max_edges, long long t, int n, unsigned *sync,
+                         cudaStream_t st) {
+    const size_t smem = s.nobj > 0 ? ib_smem_bytes(max_nodes, max_edges) : 0;
+    switch (s.prec) {
+        case LBIB_POP_F32: return launch_steps_v<float>(s, smem, t, n, sync, st);
+        case LBIB_POP_F16S: return launch_steps_v<__half>(s, smem, t, n, sync, st);
+        default: return launch_steps_v<__nv_bfloat16>(s, smem, t, n, sync, st);
+    }
+}
+
+}  // namespace lbib
