@@ -511,13 +511,11 @@ lbib_status lbib_template_create(lbib_sim *s, int tid, const double *xyz, int nn
     const size_t es = edge_stride(T);
     std::vector<int32_t> edge(10 * es, 0);  // quads (4 es), rest state (4 es), rest areas of the owned triangles (2 es)
     std::vector<char> owned(nt, 0);
-    // device records in the conflict-free evaluation order of each kind
-    for (int j = 0; j < nt; ++j) {
-        const int t = T.tri_order[j];
-        for (int k = 0; k < 3; ++k) tri4[4 * j + k] = T.tri[3 * t + k];
-        tri4[4 * j + 3] = fbits(T.S0[t]);
+    for (int t = 0; t < nt; ++t) {
+        for (int k = 0; k < 3; ++k) tri4[4 * t + k] = T.tri[3 * t + k];
+        tri4[4 * t + 3] = fbits(T.S0[t]);
     }
-    // edge e is (b, c) of bending quad e = (a, b, c, d): one record per edge
+    // edge records in the conflict-free evaluation order: edge e is (b, c) of bending quad e = (a, b, c, d): one record per edge
     // carries both (the stretching and the bending of that edge)
     for (int j = 0; j < T.ne; ++j) {
         const int e = T.quad_order[j];

@@ -74,7 +74,7 @@ enum : uint32_t {
 
 // Element lists of one template (device), all node ids local to an object:
 //   tri:        (a, b, c, rest area S0 as float bits), inward-ordered, in the
-//               bank-aware evaluation order of topology.cpp (read-outs)
+//               mesh's order (read-outs)
 struct TplDev {
     int nn, nt;
     const int4 *tri;

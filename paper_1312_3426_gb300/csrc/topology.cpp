@@ -163,7 +163,6 @@ bool build_template(const double *xyz, int nn, const int32_t *tris, int nt, cons
     }
 
     T.quad_order = conflict_free_order(T.quads, 4, 32);
-    T.tri_order = conflict_free_order(T.tri, 3, 32);
     return true;
 }
 

@@ -17,10 +17,10 @@ struct Topology {
     std::vector<int> quads;                   // [ne][4] (a, b, c, d); edge e is (b, c) of quad e
     std::vector<double> L0, theta0, S0;       // [ne], [ne], [nt]
     double Sg0 = 0.0, V0 = 0.0;
-    // device evaluation order of each element list (edges go with their
-    // quads): consecutive groups of 32 elements touch pairwise-different
-    // nodes where possible, so the lanes of a warp load different banks
-    std::vector<int> quad_order, tri_order;
+    // device evaluation order of the edges (with their quads): consecutive
+    // groups of 32 touch pairwise-different nodes where possible, so the lanes
+    // of a warp load different banks
+    std::vector<int> quad_order;
     // walks around the nodes (see ring_walks)
     std::vector<int> slots;       // [n_slots][3]: node or -1, first record, number of records
     std::vector<uint32_t> rings;  // [n records][4]: q | start flag, edge (v,q), edge (p,q), triangle
