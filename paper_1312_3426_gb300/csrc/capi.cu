@@ -3,6 +3,8 @@
 // sticky error model.  Host code only; the kernels live in fluid.cu, ib.cu
 // and batch.cu.
 #include <cuda_runtime.h>
+#include <sys/mman.h>
+#include <unistd.h>
 
 #include <algorithm>
 #include <atomic>
@@ -11,6 +13,7 @@
 #include <cstring>
 #include <initializer_list>
 #include <string>
+#include <thread>
 #include <vector>
 
 #include "lbib.h"
@@ -132,20 +135,97 @@ lbib_status sim_check_status(lbib_sim *s) {
     return apply_status(s, *s->status_pinned);
 }
 
-lbib_status sim_download_nodes(lbib_sim *s) {
-    if (!s->dev_newer) return LBIB_OK;
+// Device memory for the time of one transfer: the population buffer that the
+// next step overwrites in every fluid cell before anything reads it.  None
+// where it is too small, or beside obstacles, whose cells no step writes.
+// (cudaMallocAsync gives its pages back at each synchronisation and took 160
+// of the 200 us of a velocity read-out at 90x50x50.)
+static void *transfer_scratch(lbib_sim *s, size_t bytes) {
+    if (s->solid_mem || bytes > (size_t)NQ * s->d.nfp * pop_elem_bytes(s->p.precision)) return nullptr;
+    return s->d.pop[(s->t + 1) & 1];
+}
+
+// Faults the pages of a large read-out's destination in beside the wait for
+// the device: a fresh array costs more in page faults than the copy takes
+// (400 MB: 16.5 ms with the copy, 3.6 without).  Contents stay, only whole pages
+// inside the range are touched, and where it is refused the copy faults.
+class Prefault {
+   public:
+    Prefault(void *p, size_t bytes) {
+        if (!p || bytes < MIN_BYTES) return;
+        const size_t page = (size_t)sysconf(_SC_PAGESIZE), a = align_up((size_t)p, page);
+        const size_t e = ((size_t)p + bytes) / page * page;
+        if (e <= a) return;
+        const size_t part = align_up((e - a + THREADS - 1) / THREADS, page);
+        for (int i = 0; i < THREADS && a + i * part < e; ++i) {
+            const size_t lo = a + i * part, n = std::min(part, e - lo);
+            try {
+                th_[i] = std::thread([lo, n] { madvise((void *)lo, n, 23 /* MADV_POPULATE_WRITE */); });
+            } catch (const std::exception &) {
+                return;  // no thread to be had
+            }
+        }
+    }
+    ~Prefault() { join(); }
+    void join() {
+        for (std::thread &t : th_)
+            if (t.joinable()) t.join();
+    }
+
+   private:
+    static constexpr size_t MIN_BYTES = 8 << 20;
+    static constexpr int THREADS = 4;
+    std::thread th_[THREADS];
+};
+
+// Node states from which the conversion between the FP64 host layout and the
+// FP32 pairs runs on the device (host loops take 5 ns a node and back, a
+// kernel and its copies 15 us).
+constexpr int NODES_ON_DEVICE = 4096;
+
+// Device node state -> FP64 positions and velocities [nn][3] (either may be null).
+static lbib_status download_nodes(lbib_sim *s, double *X, double *V) {
     const int nn = s->nn_total;
-    std::vector<float> st(12 * (size_t)nn);  // Xh, Xl, Vh, Vl, each [3][nn]
+    const size_t n3 = 3 * (size_t)nn;
+    double *tmp = nn >= NODES_ON_DEVICE ? (double *)transfer_scratch(s, 2 * n3 * 8) : nullptr;
+    if (tmp) {
+        LBIB_CUDA(s, launch_pack_nodes(s->d, tmp, s->stream), "nodes D2H");
+        if (X) LBIB_CUDA(s, cudaMemcpyAsync(X, tmp, n3 * 8, cudaMemcpyDeviceToHost, s->stream), "nodes D2H");
+        if (V) LBIB_CUDA(s, cudaMemcpyAsync(V, tmp + n3, n3 * 8, cudaMemcpyDeviceToHost, s->stream), "nodes D2H");
+        LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "nodes D2H");
+        return LBIB_OK;
+    }
+    std::vector<float> st(4 * n3);  // Xh, Xl, Vh, Vl, each [3][nn]
     LBIB_CUDA(s, cudaMemcpyAsync(st.data(), s->dnodes, st.size() * 4, cudaMemcpyDeviceToHost, s->stream), "nodes D2H");
     LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "nodes D2H");
-    const size_t n3 = 3 * (size_t)nn;
     for (int i = 0; i < nn; ++i)
         for (int k = 0; k < 3; ++k) {
             const size_t j = (size_t)k * nn + i;
-            s->hX[3 * (size_t)i + k] = (double)st[j] + (double)st[n3 + j];
-            s->hV[3 * (size_t)i + k] = (double)st[2 * n3 + j] + (double)st[3 * n3 + j];
+            if (X) X[3 * (size_t)i + k] = (double)st[j] + (double)st[n3 + j];
+            if (V) V[3 * (size_t)i + k] = (double)st[2 * n3 + j] + (double)st[3 * n3 + j];
         }
+    return LBIB_OK;
+}
+
+// Brings the host mirror up to date, but for what the caller has set since
+// the last step.
+lbib_status sim_download_nodes(lbib_sim *s) {
+    if (!s->dev_newer) return LBIB_OK;
+    if (s->n_replaced == 0) {
+        const lbib_status r = download_nodes(s, s->hX.data(), s->hV.data());
+        if (r != LBIB_OK) return r;
+    } else {
+        std::vector<double> X(s->hX.size()), V(s->hV.size());
+        const lbib_status r = download_nodes(s, X.data(), V.data());
+        if (r != LBIB_OK) return r;
+        for (size_t o = 0; o < s->objs.size(); ++o) {
+            const size_t a = 3 * (size_t)s->objs[o].first, n = 3 * (size_t)s->objs[o].nn;
+            if (!(s->replaced[o] & 1)) std::copy_n(&X[a], n, &s->hX[a]);
+            if (!(s->replaced[o] & 2)) std::copy_n(&V[a], n, &s->hV[a]);
+        }
+    }
     s->dev_newer = false;
+    s->n_replaced = 0;
     return LBIB_OK;
 }
 
@@ -241,6 +321,13 @@ lbib_status sim_upload(lbib_sim *s) {
     }
     if (s->host_newer) {
         const int nn = s->nn_total;
+        if (s->dev_newer && s->n_replaced < 2 * (int)s->objs.size()) {
+            const lbib_status r = sim_download_nodes(s);
+            if (r != LBIB_OK) return r;
+        }
+        s->dev_newer = false;  // every object has new positions and velocities
+        s->n_replaced = 0;
+        bool owners = s->d.nn_total != nn;  // node_obj must be rebuilt
         if (nn > s->dev_nn_cap) {
             if (s->dnodes) cudaFree(s->dnodes);
             s->dnodes = nullptr;
@@ -248,25 +335,17 @@ lbib_status sim_upload(lbib_sim *s) {
             LBIB_CUDA(s, cudaMalloc(&s->dnodes, 16 * (size_t)nn * 4), "node state");
             s->dev_nn_cap = nn;
             s->node_bytes = 16 * (size_t)nn * 4;
+            owners = true;
         }
-        // FP64 host values split exactly into hi + lo FP32 pairs (48 bits);
-        // the membrane forces are recomputed before they are used
-        std::vector<float> st(16 * (size_t)nn, 0.f);
         const size_t n3 = 3 * (size_t)nn;
-        for (int i = 0; i < nn; ++i)
-            for (int k = 0; k < 3; ++k) {
-                const size_t j = (size_t)k * nn + i;
-                const double x = s->hX[3 * (size_t)i + k], v = s->hV[3 * (size_t)i + k];
-                st[j] = (float)x;
-                st[n3 + j] = (float)(x - (double)st[j]);
-                st[2 * n3 + j] = (float)v;
-                st[3 * n3 + j] = (float)(v - (double)st[2 * n3 + j]);
-            }
-        int32_t *owner = (int32_t *)(st.data() + 5 * n3);
-        for (int o = 0; o < (int)s->objs.size(); ++o)
-            for (int p = 0; p < s->objs[o].nn; ++p) owner[s->objs[o].first + p] = o;
-        LBIB_CUDA(s, cudaMemcpyAsync(s->dnodes, st.data(), st.size() * 4, cudaMemcpyHostToDevice, s->stream), "nodes H2D");
-        LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "nodes H2D");
+        if (owners) {
+            std::vector<int32_t> owner(nn);
+            for (int o = 0; o < (int)s->objs.size(); ++o)
+                std::fill_n(owner.begin() + s->objs[o].first, s->objs[o].nn, o);
+            LBIB_CUDA(s, cudaMemcpyAsync(s->dnodes + 5 * n3, owner.data(), (size_t)nn * 4, cudaMemcpyHostToDevice, s->stream),
+                      "nodes H2D");
+            LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "nodes H2D");
+        }
         s->d.Xh = s->dnodes;
         s->d.Xl = s->dnodes + n3;
         s->d.Vh = s->dnodes + 2 * n3;
@@ -274,6 +353,29 @@ lbib_status sim_upload(lbib_sim *s) {
         s->d.Fel = s->dnodes + 4 * n3;
         s->d.node_obj = (const int *)(s->dnodes + 5 * n3);
         s->d.nn_total = nn;
+        // FP64 host values split exactly into hi + lo FP32 pairs (48 bits);
+        // the membrane forces are recomputed before they are used
+        double *tmp = nn >= NODES_ON_DEVICE ? (double *)transfer_scratch(s, 2 * n3 * 8) : nullptr;
+        if (tmp) {
+            LBIB_CUDA(s, cudaMemcpyAsync(tmp, s->hX.data(), n3 * 8, cudaMemcpyHostToDevice, s->stream), "nodes H2D");
+            LBIB_CUDA(s, cudaMemcpyAsync(tmp + n3, s->hV.data(), n3 * 8, cudaMemcpyHostToDevice, s->stream), "nodes H2D");
+            LBIB_CUDA(s, launch_unpack_nodes(s->d, tmp, s->stream), "nodes H2D");
+            LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "nodes H2D");
+        } else {
+            std::vector<float> st(5 * n3, 0.f);
+            for (int i = 0; i < nn; ++i)
+                for (int k = 0; k < 3; ++k) {
+                    const size_t j = (size_t)k * nn + i;
+                    const double x = s->hX[3 * (size_t)i + k], v = s->hV[3 * (size_t)i + k];
+                    st[j] = (float)x;
+                    st[n3 + j] = (float)(x - (double)st[j]);
+                    st[2 * n3 + j] = (float)v;
+                    st[3 * n3 + j] = (float)(v - (double)st[2 * n3 + j]);
+                }
+            LBIB_CUDA(s, cudaMemcpyAsync(s->dnodes, st.data(), st.size() * 4, cudaMemcpyHostToDevice, s->stream),
+                      "nodes H2D");
+            LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "nodes H2D");
+        }
         s->host_newer = false;
         s->fel_valid = false;
         // the velocity samples must be valid at the (new) node corners, and
@@ -777,8 +879,12 @@ static lbib_status set_node_array(lbib_sim *s, int oid, const double *src, int n
     LBIB_GUARD(s);
     if (oid < 0 || oid >= (int)s->objs.size()) return fail(s, LBIB_ERR_ID, "unknown object id");
     if (!src || n != s->objs[oid].nn) return fail(s, LBIB_ERR_ARG, "node count must equal the template's");
-    lbib_status r = sim_download_nodes(s);
-    if (r != LBIB_OK) return r;
+    if (s->dev_newer) {  // the rest of the mirror stays out of date until it is needed
+        const char bit = positions ? 1 : 2;
+        if (s->n_replaced == 0) s->replaced.assign(s->objs.size(), 0);
+        if (!(s->replaced[oid] & bit)) s->n_replaced++;
+        s->replaced[oid] |= bit;
+    }
     std::vector<double> &dst = positions ? s->hX : s->hV;
     std::memcpy(&dst[3 * (size_t)s->objs[oid].first], src, 3 * (size_t)n * 8);
     s->host_newer = true;
@@ -951,8 +1057,16 @@ lbib_status lbib_read_nodes(lbib_sim *s, int oid, double *xyz, double *v, int64_
     const int64_t first = oid < 0 ? 0 : s->objs[oid].first;
     const int64_t n = oid < 0 ? s->nn_total : s->objs[oid].nn;
     if (cap < n) return fail(s, LBIB_ERR_ARG, "capacity too small");
+    Prefault px(xyz, 3 * (size_t)n * 8), pv(v, 3 * (size_t)n * 8);
     lbib_status r = sim_check_status(s);
     if (r != LBIB_OK) return r;
+    // all nodes: straight from the device (one object: through the mirror,
+    // which the reads of the other objects then find up to date)
+    if (oid < 0 && s->dev_newer && s->n_replaced == 0) {
+        px.join();
+        pv.join();
+        return download_nodes(s, xyz, v);
+    }
     r = sim_download_nodes(s);
     if (r != LBIB_OK) return r;
     if (xyz) std::memcpy(xyz, &s->hX[3 * first], 3 * n * 8);
@@ -965,16 +1079,19 @@ static lbib_status read_fields(lbib_sim *s, float *u, float *rho, int64_t cap) {
     if (!s->fluid_ready) return fail(s, LBIB_ERR_STATE, "fluid not initialised");
     const int64_t ncell = (int64_t)s->p.nx * s->p.ny * s->p.nz;
     if (cap < (u ? 3 : 1) * ncell) return fail(s, LBIB_ERR_ARG, "capacity too small");
+    const size_t bytes = (size_t)(u ? 3 : 1) * ncell * 4;
+    Prefault pages(u ? u : rho, bytes);
     lbib_status r = sim_check_status(s);
     if (r != LBIB_OK) return r;
-    const size_t bytes = (size_t)(u ? 3 : 1) * ncell * 4;
-    float *tmp = nullptr;
-    LBIB_CUDA(s, cudaMallocAsync((void **)&tmp, bytes, s->stream), "read-out buffer");
+    float *tmp = (float *)transfer_scratch(s, bytes);
+    const bool own = tmp == nullptr;
+    if (own) LBIB_CUDA(s, cudaMallocAsync((void **)&tmp, bytes, s->stream), "read-out buffer");
     cudaError_t e = cudaMemsetAsync(tmp, 0, bytes, s->stream);
     if (e == cudaSuccess)
         e = launch_fields(s->d, (int)(s->t & 1), s->gmode, u ? tmp : nullptr, u ? nullptr : tmp, 0, s->stream);
+    pages.join();
     if (e == cudaSuccess) e = cudaMemcpyAsync(u ? u : rho, tmp, bytes, cudaMemcpyDeviceToHost, s->stream);
-    cudaFreeAsync(tmp, s->stream);
+    if (own) cudaFreeAsync(tmp, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "read-out");
     if (rho && s->p.walls_y) {
@@ -1102,13 +1219,14 @@ lbib_status lbib_fluid_mass(lbib_sim *s, double *mass) {
     LBIB_GUARD(s);
     if (!mass) return fail(s, LBIB_ERR_ARG, "null output");
     if (!s->fluid_ready) return fail(s, LBIB_ERR_STATE, "fluid not initialised");
-    double *acc = nullptr;
-    LBIB_CUDA(s, cudaMallocAsync((void **)&acc, 8, s->stream), "mass buffer");
+    double *acc = (double *)transfer_scratch(s, 8);
+    const bool own = acc == nullptr;
+    if (own) LBIB_CUDA(s, cudaMallocAsync((void **)&acc, 8, s->stream), "mass buffer");
     cudaError_t e = cudaMemsetAsync(acc, 0, 8, s->stream);
     double dev = 0.0;
     if (e == cudaSuccess) e = launch_mass(s->d, (int)(s->t & 1), acc, s->stream);
     if (e == cudaSuccess) e = cudaMemcpyAsync(&dev, acc, 8, cudaMemcpyDeviceToHost, s->stream);
-    cudaFreeAsync(acc, s->stream);
+    if (own) cudaFreeAsync(acc, s->stream);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s->stream);
     if (e != cudaSuccess) return cuda_fail(s, e, "mass");
     *mass = (double)(s->d.nf - s->d.nsolid) * s->p.rho0 + dev;

@@ -318,6 +318,8 @@ cudaError_t launch_nodes(const SimDev &s, int par, int threads, cudaStream_t st,
 cudaError_t launch_repulsion(const SimDev &s, int max_nodes, cudaStream_t st);
 // oid >= 0: one object into out[14]; oid < 0: every object into out[nobj][14]
 cudaError_t launch_mark_all(const SimDev &s, cudaStream_t st);
+cudaError_t launch_pack_nodes(const SimDev &s, double *out, cudaStream_t st);
+cudaError_t launch_unpack_nodes(const SimDev &s, const double *in, cudaStream_t st);
 cudaError_t launch_analyze(const SimDev &s, int oid, double *out, cudaStream_t st);
 
 }  // namespace lbib

@@ -37,6 +37,8 @@ struct lbib_sim {
     std::vector<double> hX, hV;  // host mirror of node state, [nn][3]
     bool host_newer = false;     // host mirror changed since the last upload
     bool dev_newer = false;      // device state advanced since the last download
+    std::vector<char> replaced;  // per object, while dev_newer: 1 positions, 2 velocities set since
+    int n_replaced = 0;          // set bits of it (0: not in use)
     bool tables_dirty = false;   // object/template tables need an upload
     float *dnodes = nullptr;     // Xh, Xl, Vh, Vl, Fel, each [3][nn_total], then node_obj [nn_total]
     int dev_nn_cap = 0;
