@@ -76,17 +76,14 @@ __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>())
     if (f < s.nf) fluid_pair<T, MODE_PLAIN>(s, (int)(t & 1), f, step_seed(t));
 }
 
-// NT nodes per work item (the plan's node chunk); 64 registers, a full
-// SM of threads (the small spill costs less than the fifth wave of the
-// 80-register form: 0.317 against 0.318 ms per step for 64 channels)
+// NT nodes per work item (the plan's node chunk), two threads each, as in k_nodes
 template <int NT>
-__global__ void __launch_bounds__(NT, 1024 / NT)
+__global__ void __launch_bounds__(2 * NT, 512 / NT)
     k_batch_nodes(const SimDev *__restrict__ sims, const long long *__restrict__ t_base, int step_off,
                   const int2 *__restrict__ items) {
     const int2 it = items[blockIdx.x];  // (simulation, first node)
     const SimDev &s = sims[it.x];
-    const int i = it.y + (int)threadIdx.x;
-    if (i < s.nn_total) node_step<MODE_PLAIN>(s, i, (int)((t_base[it.x] + step_off) & 1));
+    node_step<MODE_PLAIN>(s, it.y + (int)(threadIdx.x >> 1), (int)((t_base[it.x] + step_off) & 1));
 }
 
 template <bool EG>
@@ -370,10 +367,10 @@ static cudaError_t enqueue_steps(cudaStream_t st, int step_off, int k) {
         const int off = step_off + j;
         if (g_plan.n_nd) {
             switch (g_plan.nthreads) {
-                case 32: k_batch_nodes<32><<<g_plan.n_nd, 32, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
-                case 64: k_batch_nodes<64><<<g_plan.n_nd, 64, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
-                case 128: k_batch_nodes<128><<<g_plan.n_nd, 128, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
-                default: k_batch_nodes<256><<<g_plan.n_nd, 256, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
+                case 32: k_batch_nodes<32><<<g_plan.n_nd, 64, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
+                case 64: k_batch_nodes<64><<<g_plan.n_nd, 128, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
+                case 128: k_batch_nodes<128><<<g_plan.n_nd, 256, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
+                default: k_batch_nodes<256><<<g_plan.n_nd, 512, 0, st>>>(g_plan.d_sims, g_plan.d_t, off, nd); break;
             }
             if ((e = cudaGetLastError()) != cudaSuccess) break;
             if ((e = cudaEventRecord(g_plan.ev_nodes, st)) != cudaSuccess) break;

@@ -29,12 +29,12 @@ __global__ void __launch_bounds__(1024, 1) k_membrane_groups(SimDev s, int T, in
     membrane_object<false>(s, o, ib_smem + (size_t)g * group_floats, tm);
 }
 
-// NT nodes per block (LBIB_TUNE_NODE_THREADS: 32, 64, 128 or 256); EARLY:
-// the instantiation for an early (programmatic dependent) launch
+// NT nodes per block (LBIB_TUNE_NODE_THREADS: 32, 64, 128 or 256), two threads
+// each; 64 registers, so 512 nodes in flight per SM.  EARLY: the instantiation
+// for an early (programmatic dependent) launch
 template <int NT, bool EARLY>
-__global__ void __launch_bounds__(NT, 1024 / NT) k_nodes(SimDev s, int par) {
-    const int i = blockIdx.x * NT + threadIdx.x;
-    if (i < s.nn_total) node_step<EARLY ? MODE_EARLY : MODE_PLAIN>(s, i, par);
+__global__ void __launch_bounds__(2 * NT, 512 / NT) k_nodes(SimDev s, int par) {
+    node_step<EARLY ? MODE_EARLY : MODE_PLAIN>(s, (int)(blockIdx.x * NT + (threadIdx.x >> 1)), par);
 }
 
 bool membrane_in_global(int max_nodes, int max_edges, int cluster) {
@@ -105,18 +105,18 @@ cudaError_t launch_membrane(const SimDev &s, int max_nodes, int max_edges, int c
     return cudaLaunchKernelEx(&cfg, global ? k_membrane<true> : k_membrane<false>, s);
 }
 
-cudaError_t launch_nodes(const SimDev &s, int par, int threads, cudaStream_t st, bool pdl) {
+cudaError_t launch_nodes(const SimDev &s, int par, int nodes, cudaStream_t st, bool pdl) {
     if (s.nn_total == 0) return cudaSuccess;
-    const unsigned blocks = (unsigned)((s.nn_total + threads - 1) / threads);
-    switch (threads * 2 + (pdl ? 1 : 0)) {
-        case 64: return launch_dep(k_nodes<32, false>, blocks, 32, st, false, s, par);
-        case 65: return launch_dep(k_nodes<32, true>, blocks, 32, st, true, s, par);
-        case 128: return launch_dep(k_nodes<64, false>, blocks, 64, st, false, s, par);
-        case 129: return launch_dep(k_nodes<64, true>, blocks, 64, st, true, s, par);
-        case 256: return launch_dep(k_nodes<128, false>, blocks, 128, st, false, s, par);
-        case 257: return launch_dep(k_nodes<128, true>, blocks, 128, st, true, s, par);
-        case 512: return launch_dep(k_nodes<256, false>, blocks, 256, st, false, s, par);
-        case 513: return launch_dep(k_nodes<256, true>, blocks, 256, st, true, s, par);
+    const unsigned blocks = (unsigned)((s.nn_total + nodes - 1) / nodes);
+    switch (nodes * 2 + (pdl ? 1 : 0)) {
+        case 64: return launch_dep(k_nodes<32, false>, blocks, 64, st, false, s, par);
+        case 65: return launch_dep(k_nodes<32, true>, blocks, 64, st, true, s, par);
+        case 128: return launch_dep(k_nodes<64, false>, blocks, 128, st, false, s, par);
+        case 129: return launch_dep(k_nodes<64, true>, blocks, 128, st, true, s, par);
+        case 256: return launch_dep(k_nodes<128, false>, blocks, 256, st, false, s, par);
+        case 257: return launch_dep(k_nodes<128, true>, blocks, 256, st, true, s, par);
+        case 512: return launch_dep(k_nodes<256, false>, blocks, 512, st, false, s, par);
+        case 513: return launch_dep(k_nodes<256, true>, blocks, 512, st, true, s, par);
         default: return cudaErrorInvalidValue;
     }
 }

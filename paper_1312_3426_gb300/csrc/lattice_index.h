@@ -69,13 +69,13 @@ LBIB_HD void lattice_coord(float hi, float lo, int &i0, float &w) {
     w = fr;
 }
 
-// The 8 interpolation corners of a point: corner k = (dx, dy, dz) =
-// (k & 1, k >> 1 & 1, k >> 2 & 1) is lattice node (i0 + dx, j0 + dy,
-// k0 + dz) with trilinear weight w[k] (the volume of the box between the
-// point and the diagonally opposite corner); f[k] = -1 on a solid row.
+// The 4 interpolation corners of a point on one side in x: corner k =
+// (dy, dz) = (k & 1, k >> 1) is lattice node (i0 + dx, j0 + dy, k0 + dz) with
+// trilinear weight w[k] (the volume of the box between the point and the
+// diagonally opposite corner); f[k] = -1 on a solid row.
 template <class D>
-LBIB_HD void corner_cells(const D &g, float xh, float xl, float yh, float yl, float zh, float zl, int (&f)[8],
-                          float (&w)[8]) {
+LBIB_HD void corner_cells_side(const D &g, float xh, float xl, float yh, float yl, float zh, float zl, int dx,
+                               int (&f)[4], float (&w)[4]) {
     int ix, iy, iz;
     float wx, wy, wz;
     lattice_coord(xh, xl, ix, wx);
@@ -95,13 +95,36 @@ LBIB_HD void corner_cells(const D &g, float xh, float xl, float yh, float yl, fl
         cy0 = wrapi(iy, g.ny);
         cy1 = cy0 + 1 == g.ny ? 0 : cy0 + 1;
     }
+    const int cx = dx ? cx1 : cx0;
+    const float wxd = dx ? wx : 1.f - wx;
 #if defined(__CUDACC__)
 #pragma unroll
 #endif
-    for (int k = 0; k < 8; ++k) {
-        const int dx = k & 1, dy = (k >> 1) & 1, dz = (k >> 2) & 1;
-        f[k] = (dy ? in1 : in0) ? (dx ? cx1 : cx0) + g.nx * ((dy ? cy1 : cy0) + g.nyf * (dz ? cz1 : cz0)) : -1;
-        w[k] = (dx ? wx : 1.f - wx) * (dy ? wy : 1.f - wy) * (dz ? wz : 1.f - wz);
+    for (int k = 0; k < 4; ++k) {
+        const int dy = k & 1, dz = k >> 1;
+        f[k] = (dy ? in1 : in0) ? cx + g.nx * ((dy ? cy1 : cy0) + g.nyf * (dz ? cz1 : cz0)) : -1;
+        w[k] = wxd * (dy ? wy : 1.f - wy) * (dz ? wz : 1.f - wz);
+    }
+}
+
+// All 8: corner k = (dx, dy, dz) = (k & 1, k >> 1 & 1, k >> 2).
+template <class D>
+LBIB_HD void corner_cells(const D &g, float xh, float xl, float yh, float yl, float zh, float zl, int (&f)[8],
+                          float (&w)[8]) {
+#if defined(__CUDACC__)
+#pragma unroll
+#endif
+    for (int dx = 0; dx < 2; ++dx) {
+        int fs[4];
+        float ws[4];
+        corner_cells_side(g, xh, xl, yh, yl, zh, zl, dx, fs, ws);
+#if defined(__CUDACC__)
+#pragma unroll
+#endif
+        for (int k = 0; k < 4; ++k) {
+            f[2 * k + dx] = fs[k];
+            w[2 * k + dx] = ws[k];
+        }
     }
 }
 

@@ -6,7 +6,7 @@
 // a step for one sphere in a 40x20x20 channel, 7 of them between kernels, and
 // the host enqueues no faster than 11 us a step.  Here one cooperative launch
 // runs all steps of a call, with two barriers over its blocks in each:
-//   node update    32 nodes per warp, spread over all blocks (on one SM the
+//   node update    16 nodes per warp, spread over all blocks (on one SM the
 //                  scattered gathers and reductions of a level-3 cell's 642
 //                  nodes take 7 us, at about one sector a cycle);
 //   [barrier]
@@ -83,8 +83,8 @@ __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, l
         const int par = (int)(t & 1);
         if (k > 0 && !steps_wait(s, done, blocks * (unsigned)k)) return;
         if (nobj > 0) {
-            for (int i = 32 * (int)((threadIdx.x >> 5) * blocks + blockIdx.x); i < s.nn_total; i += THREADS * (int)blocks)
-                if (i + (int)(threadIdx.x & 31) < s.nn_total) node_step<MODE_MANY>(s, i + (int)(threadIdx.x & 31), par);
+            for (int i = 16 * (int)((threadIdx.x >> 5) * blocks + blockIdx.x); i < s.nn_total; i += THREADS / 2 * (int)blocks)
+                node_step<MODE_MANY>(s, i + (int)((threadIdx.x & 31) >> 1), par);
             steps_signal(nodes_done);
             if (!steps_wait(s, nodes_done, blocks * (unsigned)(k + 1))) return;
         }
