@@ -135,30 +135,17 @@ cudaError_t launch_nodes(const SimDev &s, int par, int nodes, cudaStream_t st, b
 //                 all of j's nodes; the pair force goes to i's node directly
 //                 and to j's node through a shared-memory sum, both added
 //                 to Fel with global atomics.
+// (Steps of small simulations: repel_object in ib_core.cuh.)
 // Separations are formed as (hi_i - hi_j) + (lo_i - lo_j), exact in the
 // leading part for nearby nodes, so the force does not lose digits at
 // large coordinates.
-
-__device__ __forceinline__ int image_shift(float ci, float cj, int L) {
-    return (int)rintf((ci - cj) / (float)L);  // j + shift * L is the image nearest to i
-}
 
 __global__ void __launch_bounds__(256) k_rep_pairs(SimDev s) {
     const int i = blockIdx.y;
     const int j = blockIdx.x * blockDim.x + threadIdx.x;
     if (j <= i || j >= s.nobj) return;
-    const float *A = s.aabb + 8 * i, *B = s.aabb + 8 * j;
-    const int L[3] = {s.nx, s.ny, s.nz};
     int k3[3];
-    bool close = true;
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        const bool periodic = k != 1 || !s.walls;
-        k3[k] = periodic ? image_shift(0.5f * (A[k] + A[3 + k]), 0.5f * (B[k] + B[3 + k]), L[k]) : 0;
-        const float sh = (float)(k3[k] * L[k]);
-        close = close && (B[k] + sh < A[3 + k] + s.rep_rc) && (A[k] < B[3 + k] + sh + s.rep_rc);
-    }
-    if (!close) return;
+    if (!close_objects(s, i, j, k3)) return;
     const unsigned slot = atomicAdd(s.npairs, 1u);
     if (slot < (unsigned)s.pair_cap)
         s.pairs[slot] = make_int4(i | (j << 16), k3[0], k3[1], k3[2]);  // nobj <= 65535

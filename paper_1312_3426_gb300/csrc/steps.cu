@@ -6,7 +6,7 @@
 // a step for one sphere in a 40x20x20 channel, 7 of them between kernels, and
 // the host enqueues no faster than 11 us a step.  Here one cooperative launch
 // runs all steps of a call, with two barriers over its blocks in each:
-//   node update    16 nodes per warp, spread over all blocks (on one SM the
+//   node update    8 nodes per warp, spread over all blocks (on one SM the
 //                  scattered gathers and reductions of a level-3 cell's 642
 //                  nodes take 7 us, at about one sector a cycle);
 //   [barrier]
@@ -21,7 +21,7 @@
 // sets ST_TIMEOUT and the block leaves.  What another block writes during the
 // launch is read through the L2 (populations, velocity samples, mask, forces,
 // and the positions of an object by its membrane block); a node's own state
-// stays with its thread.
+// stays with its warp.
 #include "fluid_core.cuh"
 #include "ib_core.cuh"
 
@@ -74,7 +74,7 @@ __device__ __forceinline__ void steps_signal(unsigned *c) {
 template <typename T, bool PAIR, bool BC>
 __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, long long t0, int n, unsigned *sync) {
     constexpr int THREADS = STEPS_THREADS<T, PAIR>, CELLS = PAIR ? 2 * THREADS : THREADS;
-    unsigned *nodes_done = sync, *done = sync + 32;
+    unsigned *nodes_done = sync, *boxes_done = sync + 16, *done = sync + 32;
     const unsigned blocks = gridDim.x;
     const int nobj = s.nobj, b = (int)blockIdx.x, nfluid = (int)blocks - nobj;
     const int tiles = (s.nf + CELLS - 1) / CELLS;
@@ -83,13 +83,19 @@ __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, l
         const int par = (int)(t & 1);
         if (k > 0 && !steps_wait(s, done, blocks * (unsigned)k)) return;
         if (nobj > 0) {
-            for (int i = 16 * (int)((threadIdx.x >> 5) * blocks + blockIdx.x); i < s.nn_total; i += THREADS / 2 * (int)blocks)
-                node_step<MODE_MANY>(s, i + (int)((threadIdx.x & 31) >> 1), par);
+            constexpr int L = NODE_LANES<MODE_MANY>;
+            for (int i = 32 / L * (int)((threadIdx.x >> 5) * blocks + blockIdx.x); i < s.nn_total; i += THREADS / L * (int)blocks)
+                node_step<MODE_MANY>(s, i + (int)(threadIdx.x & 31) / L, par);
             steps_signal(nodes_done);
             if (!steps_wait(s, nodes_done, blocks * (unsigned)(k + 1))) return;
         }
         if (b < nobj) {
             membrane_object<false, MODE_MANY>(s, b, steps_smem, BlockTeam());
+            if (s.rep_on) {  // the other objects' boxes
+                steps_signal(boxes_done);
+                if (!steps_wait(s, boxes_done, (unsigned)nobj * (unsigned)(k + 1))) return;
+                repel_object(s, b, steps_smem);
+            }
         } else {
             const uint32_t seed = step_seed(t);
             for (int tile = b - nobj; tile < tiles; tile += nfluid) {
@@ -145,7 +151,7 @@ static int steps_fluid_blocks(const SimDev &s) {
 // beyond (10 rounds at 160x96x96 FP32, 160x128x96 FP16) they are equal.
 bool steps_fit(const SimDev &s, int max_nodes, int max_edges) {
     const int sms = device_sms();
-    if (s.rep_on || (s.nobj > 0 && ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX)) return false;
+    if ((s.rep_on && s.nobj > REPEL_MAX_OBJECTS) || (s.nobj > 0 && ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX)) return false;
     const int tiles = steps_tiles(s);
     if (s.nobj == 0) return tiles >= 32 && tiles <= 5 * sms;
     return 2 * s.nobj <= sms && tiles <= 8 * (sms - s.nobj);
