@@ -811,12 +811,13 @@ lbib_status lbib_set_solid(lbib_sim *s, const uint8_t *mask, int64_t n) {
                 bits[f >> 5] |= 1u << (f & 31);
                 ++count;
             }
-    if (!s->solid_mem) LBIB_CUDA(s, cudaMalloc(&s->solid_mem, (size_t)d.nwords * 4), "obstacle mask");
+    if (!s->solid_mem) LBIB_CUDA(s, cudaMalloc(&s->solid_mem, (size_t)d.nwords * 8), "obstacle mask");
     LBIB_CUDA(s, cudaMemcpyAsync(s->solid_mem, bits.data(), bits.size() * 4, cudaMemcpyHostToDevice, s->stream),
               "obstacle mask");
-    LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "obstacle mask");
     d.solid = s->solid_mem;
     d.nsolid = count;
+    LBIB_CUDA(s, launch_near_bits(d, s->solid_mem + d.nwords, s->stream), "obstacle mask");
+    LBIB_CUDA(s, cudaStreamSynchronize(s->stream), "obstacle mask");
     return LBIB_OK;
 }
 
@@ -1287,7 +1288,7 @@ lbib_status lbib_info(const lbib_sim *s, int64_t out[8]) {
     out[3] = s->d.nf;
     out[4] = s->t;
     out[5] = (int64_t)(s->fluid_bytes + s->tpl_bytes + s->node_bytes + s->rep_bytes + s->edge_bytes +
-                       (s->solid_mem ? (size_t)s->d.nwords * 4 : 0));
+                       (s->solid_mem ? (size_t)s->d.nwords * 8 : 0));
     out[6] = s->p.precision;
     out[7] = fluid_kernel_kind(s->d);
     return LBIB_OK;

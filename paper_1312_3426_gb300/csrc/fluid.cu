@@ -122,6 +122,32 @@ cudaError_t launch_fluid(const SimDev &s, int par, long long t, cudaStream_t st,
     }
 }
 
+// near_bit of every cell: one of its 18 sources (periodic) is an obstacle
+__global__ void k_near_bits(SimDev s, uint32_t *near) {
+    const int f = blockIdx.x * blockDim.x + threadIdx.x;
+    bool any = false;
+    if (f < s.nf) {
+        const int x = f % s.nx, r = f / s.nx, y = r % s.nyf, z = r / s.nyf;
+        const Rows n = source_rows(s, (uint32_t)f, y, z);
+        const int xm = x == 0 ? s.nx - 1 : -1, xp = x == s.nx - 1 ? 1 - s.nx : 1;
+#pragma unroll
+        for (int i = 0; i < 3; ++i)
+#pragma unroll
+            for (int j = 0; j < 3; ++j) {
+                const int g = (int)n.row[i][j];
+                any = any || ((i != 1 || j != 1) && solid_bit(s, g));
+                if (i == 1 || j == 1) any = any || solid_bit(s, g + xm) || solid_bit(s, g + xp);
+            }
+    }
+    const uint32_t word = __ballot_sync(0xffffffffu, any);
+    if ((threadIdx.x & 31) == 0 && (f >> 5) < s.nwords) near[f >> 5] = word;
+}
+
+cudaError_t launch_near_bits(const SimDev &s, uint32_t *near, cudaStream_t st) {
+    k_near_bits<<<(s.nf + 255) / 256, 256, 0, st>>>(s, near);
+    return cudaGetLastError();
+}
+
 // ---------------------------------------------------------------- read-outs
 
 __device__ __forceinline__ int64_t full_index(const SimDev &s, int f) {

@@ -140,20 +140,41 @@ struct Raw<__nv_bfloat16> {
     }
 };
 
-// Pull the (raw) population of direction Q arriving at a cell (xm, xp: steps
-// to x - 1 and x + 1, periodic; walls not considered).  In the
-// boundary-condition variant (BC) a population coming from an obstacle cell
-// is the cell's own opposite one, as at the walls.
-template <typename T, int Q, bool BC, int MODE>
-__device__ __forceinline__ float pull(const SimDev &s, const T *__restrict__ src, size_t nfp, const Rows &n, int xm,
-                                      int xp) {
+// The cell from which population Q of a cell arrives (xm, xp: steps to x - 1
+// and x + 1, periodic; walls and obstacles not considered).
+template <int Q>
+__device__ __forceinline__ uint32_t source_cell(const Rows &n, int xm, int xp) {
     constexpr int ex = d3q19_ex(Q), ey = d3q19_ey(Q), ez = d3q19_ez(Q);
     uint32_t g = n.row[1 + ey][1 + ez];
     if constexpr (ex == 1) g += (uint32_t)xm;
     if constexpr (ex == -1) g += (uint32_t)xp;
-    if (BC && Q != 0 && s.solid && solid_bit(s, (int)g))
-        return Raw<T>::template ld<MODE>(src + (size_t)d3q19_opp(Q) * nfp + n.row[1][1]);
-    return Raw<T>::template ld<MODE>(src + (size_t)Q * nfp + g);
+    return g;
+}
+
+// Pull the (raw) population of direction Q arriving at a cell.
+template <typename T, int Q, int MODE>
+__device__ __forceinline__ float pull(const T *__restrict__ src, size_t nfp, const Rows &n, int xm, int xp) {
+    return Raw<T>::template ld<MODE>(src + (size_t)Q * nfp + source_cell<Q>(n, xm, xp));
+}
+
+// Bounce-back at obstacles: a population coming from an obstacle cell is the
+// cell's own opposite one.  As at the walls, the pulls already on the way are
+// replaced, and only warps with a cell next to an obstacle (near bits) come
+// here.  With the 18 bits of the sources asked for before each pull, the
+// kernel waited for them one after the other (fluid steps among posts:
+// 199x50x30 FP16 20.5 -> 12.3 us, 256x128x128 FP16 211 -> 98, FP32 160 -> 110).
+template <typename T, int MODE>
+__device__ __forceinline__ void bounce_obstacles(const SimDev &s, const T *__restrict__ src, size_t nfp, uint32_t f,
+                                                 const Rows &n, int xm, int xp, float (&h)[NQ]) {
+    uint32_t from = 0u;
+#define LBIB_SOURCE(q) from |= (uint32_t)solid_bit(s, (int)source_cell<q>(n, xm, xp)) << q;
+    LBIB_SOURCE(1) LBIB_SOURCE(2) LBIB_SOURCE(3) LBIB_SOURCE(4) LBIB_SOURCE(5) LBIB_SOURCE(6) LBIB_SOURCE(7)
+    LBIB_SOURCE(8) LBIB_SOURCE(9) LBIB_SOURCE(10) LBIB_SOURCE(11) LBIB_SOURCE(12) LBIB_SOURCE(13) LBIB_SOURCE(14)
+    LBIB_SOURCE(15) LBIB_SOURCE(16) LBIB_SOURCE(17) LBIB_SOURCE(18)
+#undef LBIB_SOURCE
+#pragma unroll
+    for (int q = 1; q < NQ; ++q)
+        if ((from >> q) & 1u) h[q] = Raw<T>::template ld<MODE>(src + (size_t)d3q19_opp(q) * nfp + f);
 }
 
 // Bounce-back at a wall row (the row below, EY = 1, or above, EY = -1, is
@@ -443,7 +464,7 @@ __device__ __forceinline__ void fluid_cell(const SimDev &s, int par, int fi, uin
     const T *__restrict__ src = (const T *)s.pop[par];
     T *__restrict__ dst = (T *)s.pop[par ^ 1];
     const uint32_t nfp = (uint32_t)s.nfp, f = (uint32_t)fi;
-    if (BC && s.solid && solid_bit(s, fi)) return;  // an obstacle cell holds no fluid
+    const bool obstacle = BC && s.solid && solid_bit(s, fi), near = BC && s.solid && near_bit(s, fi);
     const uint32_t r = s.div_nx.div(f);
     const uint32_t x = f - r * (uint32_t)s.nx;
     const uint32_t z = s.div_nyf.div(r);
@@ -452,11 +473,15 @@ __device__ __forceinline__ void fluid_cell(const SimDev &s, int par, int fi, uin
     const int xm = x == 0 ? s.nx - 1 : -1, xp = x == (uint32_t)s.nx - 1 ? 1 - s.nx : 1;
 
     float h[NQ];
-#define LBIB_PULL(q) h[q] = pull<T, q, BC, MODE>(s, src, nfp, n, xm, xp);
+#define LBIB_PULL(q) h[q] = pull<T, q, MODE>(src, nfp, n, xm, xp);
     LBIB_PULL(0) LBIB_PULL(1) LBIB_PULL(2) LBIB_PULL(3) LBIB_PULL(4) LBIB_PULL(5) LBIB_PULL(6)
     LBIB_PULL(7) LBIB_PULL(8) LBIB_PULL(9) LBIB_PULL(10) LBIB_PULL(11) LBIB_PULL(12) LBIB_PULL(13)
     LBIB_PULL(14) LBIB_PULL(15) LBIB_PULL(16) LBIB_PULL(17) LBIB_PULL(18)
 #undef LBIB_PULL
+    if (BC && __any_sync(__activemask(), obstacle || near)) {
+        if (obstacle) return;  // holds no fluid
+        if (near) bounce_obstacles<T, MODE>(s, src, nfp, f, n, xm, xp, h);
+    }
     const bool ylo = s.walls && y == 0, yhi = s.walls && y == (uint32_t)s.nyf - 1;
     if (__any_sync(__activemask(), ylo || yhi)) {
         if (ylo) bounce<T, 1, MODE>(src, nfp, f, h);

@@ -182,7 +182,7 @@ struct SimDev {
     int in_box[6];
     float in_u[3];
     // obstacle cells (bit per fluid cell, nwords words; null: none): solid
-    // like the wall rows
+    // like the wall rows; then as many words of near_bit
     const uint32_t *solid;
     int nsolid;
     // 16-bit storage: fluid kernel preference (0 and 1 two cells per thread
@@ -194,6 +194,10 @@ struct SimDev {
 #ifdef __CUDACC__
 __device__ __forceinline__ bool solid_bit(const SimDev &s, int f) {
     return (__ldg(s.solid + (f >> 5)) >> (f & 31)) & 1u;
+}
+// a neighbour (18 directions, periodic) is an obstacle cell
+__device__ __forceinline__ bool near_bit(const SimDev &s, int f) {
+    return (__ldg(s.solid + s.nwords + (f >> 5)) >> (f & 31)) & 1u;
 }
 #endif
 
@@ -258,6 +262,8 @@ cudaError_t launch_dep(void (*k)(KArgs...), unsigned grid, unsigned block, cudaS
 // pdl: launch with programmatic stream serialization (only right after the
 // node kernel of the same step)
 cudaError_t launch_fluid(const SimDev &s, int par, long long t, cudaStream_t st, bool pdl = false);
+// the near_bit words of the obstacle bits
+cudaError_t launch_near_bits(const SimDev &s, uint32_t *near, cudaStream_t st);
 // the kernel launch_fluid picks (lbib_info out[7]): 0 one cell per thread,
 // 1 two cells per thread, 2 warp-specialised two cells per thread
 int fluid_kernel_kind(const SimDev &s);
