@@ -328,7 +328,7 @@ LBIB_API lbib_status lbib_fluid_mass_noalloc(lbib_sim *sim, double *mass);
 /* Counts (oif_info, Sec. 5).  out[8] = n_templates, n_objects, n_nodes,
  * fluid cells, steps taken, device bytes held, precision, and the fluid
  * kernel the step uses: 0 one cell per thread; 1 two x-adjacent cells per
- * thread (even nx, no obstacles, no inlet); 2 the
+ * thread (no obstacles, no inlet); 2 the
  * warp-specialised two-cells kernel (see LBIB_TUNE_FLUID_KERNEL). */
 LBIB_API lbib_status lbib_info(const lbib_sim *sim, int64_t out[8]);
 
@@ -396,7 +396,7 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * picks 128 to 1024 by the number and size of the objects and the length of
  * the fluid update beside them; fewer threads leave more of each SM to the
  * fluid kernel).  LBIB_TUNE_FLUID_KERNEL (16-bit storage): 0
- * (default) and 1 the two-cells-per-thread kernel (where nx is even and
+ * (default) and 1 the two-cells-per-thread kernel (where
  * there are no obstacles or inlet), 2 the warp-specialised two-cells kernel
  * (a producer warp streams the populations through shared memory with bulk
  * asynchronous copies; needs nx a multiple of 8 with a row segment of at

@@ -34,7 +34,7 @@
 namespace lbib {
 
 constexpr int LBIB_BATCH_GRAPH_STEPS = 16;  // steps per captured graph
-constexpr int FLUID_GROUPS = 9;             // fluid kernel variants (see fluid_group)
+constexpr int FLUID_GROUPS = 10;            // fluid kernel variants (see fluid_group)
 
 extern __shared__ float batch_smem[];
 
@@ -63,8 +63,8 @@ __global__ void __launch_bounds__(FLUID_THREADS, 5)
     fluid_block<T, BC, MODE_PLAIN>(s, (int)(t & 1), it.y * FLUID_THREADS, step_seed(t));
 }
 
-// Even nx, plain boundaries: two cells per thread.
-template <typename T>
+// Plain boundaries, 16-bit storage: two cells per thread (ODD: nx odd).
+template <typename T, bool ODD>
 __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>())
     k_batch_fluid_pair(const SimDev *__restrict__ sims, const long long *__restrict__ t_base, int step_off,
                        const int2 *__restrict__ items, int pf) {
@@ -73,7 +73,7 @@ __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>())
     const SimDev &s = sims[it.x];
     const long long t = t_base[it.x] + step_off;
     const int f = 2 * (it.y * PAIR_THREADS + (int)threadIdx.x);
-    if (f < s.nf) fluid_pair<T, MODE_PLAIN>(s, (int)(t & 1), f, step_seed(t));
+    if (f < s.nf) fluid_pair<T, MODE_PLAIN, ODD>(s, (int)(t & 1), f, step_seed(t));
 }
 
 // NT nodes per work item (the plan's node chunk), two threads each, as in k_nodes
@@ -135,7 +135,7 @@ struct BatchPlan {
     // their defaults
     int big_threads = 0, rest_threads = 0;
     bool mauto = false;
-    int pf_cell = 0, pf_pair[2] = {};  // (pairs: 16-bit, FP32) L2 prefetch distances of the fluid launches (work items)
+    int pf_cell = 0, pf_pair = 0;  // L2 prefetch distances of the fluid launches (work items)
     cudaStream_t aux = nullptr;   // membrane kernel
     cudaStream_t aux2 = nullptr;  // membrane kernel of the smaller size class
     cudaEvent_t ev_rest = nullptr;
@@ -169,10 +169,13 @@ static BatchPlan g_plan;
 static std::mutex g_plan_mu;
 
 // Fluid kernel variant of a simulation: 2 * precision + BC (obstacles or an
-// inlet) for the one-cell-per-thread kernels; 6 + precision for the two-cells
-// kernels.
+// inlet) for the one-cell-per-thread kernels; for 16-bit storage 5 + precision
+// for the two-cells kernel, 7 + precision for that of an odd nx.  FP32 takes the
+// one-cell kernel here, with 40 warps an SM instead of 20: the boxes of a batch
+// are narrow and many, and even and odd widths share a launch (64 mixed channels
+// 309.2 us a step against 318.3, 24 channels up to 192x96x96 272.7 against 279.7).
 static int fluid_group(const lbib_sim *s) {
-    if (fluid_kernel_kind(s->d) != 0) return 6 + s->d.prec;
+    if (s->d.prec != LBIB_POP_F32 && fluid_kernel_kind(s->d) != 0) return (s->d.nx & 1 ? 7 : 5) + s->d.prec;
     return 2 * s->d.prec + (s->d.solid || s->d.in_on ? 1 : 0);
 }
 
@@ -257,8 +260,7 @@ static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStr
         int sms = 0;
         if ((e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, g_plan.device)) != cudaSuccess) return e;
         g_plan.pf_cell = fluid_prefetch(LBIB_POP_F32, 0, sms);  // as in the single-simulation launches
-        g_plan.pf_pair[0] = fluid_prefetch(LBIB_POP_F16S, 1, sms);
-        g_plan.pf_pair[1] = fluid_prefetch(LBIB_POP_F32, 1, sms);
+        g_plan.pf_pair = fluid_prefetch(LBIB_POP_F16S, 1, sms);
     }
     g_plan.max_nodes = max_nodes;
     g_plan.max_edges = max_edges;
@@ -383,7 +385,7 @@ static cudaError_t enqueue_steps(cudaStream_t st, int step_off, int k) {
             const int *n = g_plan.n_flp;
             const SimDev *ds = g_plan.d_sims;
             const long long *dt = g_plan.d_t;
-            const int p1 = g_plan.pf_cell, p2 = g_plan.pf_pair[0], p4 = g_plan.pf_pair[1];
+            const int p1 = g_plan.pf_cell, p2 = g_plan.pf_pair;
             if (n[0]) k_batch_fluid<float, false><<<n[0], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p1);
             g += n[0];
             if (n[1]) k_batch_fluid<float, true><<<n[1], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p1);
@@ -396,11 +398,13 @@ static cudaError_t enqueue_steps(cudaStream_t st, int step_off, int k) {
             g += n[4];
             if (n[5]) k_batch_fluid<__nv_bfloat16, true><<<n[5], FLUID_THREADS, 0, st>>>(ds, dt, off, g, p1);
             g += n[5];
-            if (n[6]) k_batch_fluid_pair<float><<<n[6], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p4);
+            if (n[6]) k_batch_fluid_pair<__half, false><<<n[6], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
             g += n[6];
-            if (n[7]) k_batch_fluid_pair<__half><<<n[7], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
+            if (n[7]) k_batch_fluid_pair<__nv_bfloat16, false><<<n[7], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
             g += n[7];
-            if (n[8]) k_batch_fluid_pair<__nv_bfloat16><<<n[8], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
+            if (n[8]) k_batch_fluid_pair<__half, true><<<n[8], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
+            g += n[8];
+            if (n[9]) k_batch_fluid_pair<__nv_bfloat16, true><<<n[9], PAIR_THREADS, 0, st>>>(ds, dt, off, g, p2);
         }
         if ((e = cudaGetLastError()) != cudaSuccess) break;
         if (g_plan.n_nd) e = cudaStreamWaitEvent(st, g_plan.ev_membrane, 0);

@@ -34,7 +34,7 @@ __global__ void __launch_bounds__(FLUID_THREADS, 5) k_fluid(SimDev s, uint32_t s
     fluid_block<T, BC, EARLY ? MODE_EARLY : MODE_PLAIN>(s, 0, block * FLUID_THREADS, seed);
 }
 
-// Even nx, no obstacles, no inlet: two cells per thread.  Both cells share
+// No obstacles, no inlet: two cells per thread (ODD: nx odd).  Both cells share
 // the index work and the packed FP32 instructions, so a warp of 64 cells
 // issues 557 (FP32) or 596 (16-bit) instructions; one cell per thread took
 // 651 for 32 FP32 cells.  FP32 is bound by DRAM either way (256x128x128
@@ -42,15 +42,15 @@ __global__ void __launch_bounds__(FLUID_THREADS, 5) k_fluid(SimDev s, uint32_t s
 // warp instructions, which leaves the issue slots to the membrane kernel
 // beside it), the 16-bit kernel by instructions (61.6 -> 57.6 us there and
 // 455 -> 431 at 512x256x256, 47.1 -> 38.4 M).
-template <typename T, bool EARLY>
+template <typename T, bool EARLY, bool ODD>
 __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>()) k_fluid_pair(SimDev s, uint32_t seed, int pf) {
     const int block = sweep_block(pf);
     prefetch_sources<sizeof(T), 2 * PAIR_THREADS>(s, s.pop[0], block, pf);
     const int f = 2 * (block * PAIR_THREADS + (int)threadIdx.x);
-    if (f < s.nf) fluid_pair<T, EARLY ? MODE_EARLY : MODE_PLAIN>(s, 0, f, seed);
+    if (f < s.nf) fluid_pair<T, EARLY ? MODE_EARLY : MODE_PLAIN, ODD>(s, 0, f, seed);
 }
 
-static bool pair_shape(const SimDev &s) { return (s.nx & 1) == 0 && !s.solid && !s.in_on; }
+static bool pair_shape(const SimDev &s) { return !s.solid && !s.in_on; }
 
 // The warp-specialised kernel is opt-in (LBIB_TUNE_FLUID_KERNEL = 2): on
 // a GB300 it ran slower than the two-cells kernel with L2 prefetch (0.0947
@@ -96,10 +96,11 @@ static cudaError_t launch_fluid_t(const SimDev &s, int par, uint32_t seed, int b
         std::swap(d.G[0], d.G[1]);
     }
     if (fluid_kernel_kind(s) == 1) {
-        const unsigned pblocks = (unsigned)((s.nf / 2 + PAIR_THREADS - 1) / PAIR_THREADS);
+        const unsigned pblocks = (unsigned)(((s.nf + 1) / 2 + PAIR_THREADS - 1) / PAIR_THREADS);
         const int pf = (par ? -1 : 1) * fluid_prefetch(s.prec, 1, sms);
-        if (pdl) return launch_dep(k_fluid_pair<T, true>, pblocks, PAIR_THREADS, st, true, d, seed, pf);
-        return launch_dep(k_fluid_pair<T, false>, pblocks, PAIR_THREADS, st, false, d, seed, pf);
+        auto *k = s.nx & 1 ? (pdl ? k_fluid_pair<T, true, true> : k_fluid_pair<T, false, true>)
+                           : (pdl ? k_fluid_pair<T, true, false> : k_fluid_pair<T, false, false>);
+        return launch_dep(k, pblocks, PAIR_THREADS, st, pdl, d, seed, pf);
     }
     const unsigned b = (unsigned)blocks;
     const int pf = (par ? -1 : 1) * fluid_prefetch(s.prec, 0, sms);

@@ -558,8 +558,9 @@ __device__ __forceinline__ void fluid_cell(const SimDev &s, int par, int fi, uin
 }
 
 // ------------------------------------------------------------------
-// Two cells per thread for 16-bit storage (nx even, no obstacles, no inlet).
-// A thread owns cells f and f+1 (f even, same row).  Populations of the
+// Two cells per thread (no obstacles, no inlet).
+// A thread owns cells f and f+1 (f even; in the same row when nx is even, else
+// see fluid_pair_odd).  Populations of the
 // two cells sit next to each other in every plane, so the pair is read as
 // one 32-bit word where the source is even (directions without an x
 // component, bounce-back) and as two 16-bit words at adjacent addresses
@@ -642,6 +643,25 @@ __device__ __forceinline__ void bounce2(const T *__restrict__ src, size_t nfp, u
 #pragma unroll
     for (int q = 1; q < NQ; ++q)
         if (d3q19_ey(q) == EY) P[q] = PairRaw<T>::template ld<MODE>(src + (size_t)d3q19_opp(q) * nfp, f);
+}
+
+// Odd nx: the pair of direction Q from any two cells, and bounce() where one or
+// both of them are at the wall
+template <typename T, int Q, int MODE>
+__device__ __forceinline__ typename PairRaw<T>::type pull_cells(const T *__restrict__ src, size_t nfp, const Rows &na,
+                                                                int xma, int xpa, const Rows &nb, int xmb, int xpb) {
+    return PairRaw<T>::template ld<MODE>(src + (size_t)Q * nfp, source_cell<Q>(na, xma, xpa), source_cell<Q>(nb, xmb, xpb));
+}
+template <typename T, int EY, int MODE>
+__device__ __forceinline__ void bounce_cells(const T *__restrict__ src, size_t nfp, uint32_t f, bool a, bool b,
+                                             typename PairRaw<T>::type (&P)[NQ]) {
+#pragma unroll
+    for (int q = 1; q < NQ; ++q)
+        if (d3q19_ey(q) == EY) {
+            const auto own = PairRaw<T>::template ld<MODE>(src + (size_t)d3q19_opp(q) * nfp, f);
+            if constexpr (sizeof(T) == 4) P[q] = make_float2(a ? own.x : P[q].x, b ? own.y : P[q].y);
+            else P[q] = __byte_perm(P[q], own, (a ? 0x0054u : 0x0010u) | (b ? 0x7600u : 0x3200u));
+        }
 }
 
 // The arithmetic of the two cells runs in packed FP32 instructions (sm_100
@@ -737,6 +757,13 @@ struct Cls2 {
     float2 K, R, R15, gx, gy, gz;
 };
 
+// OWN: in the order in which the one-cell kernel's sums are contracted
+template <bool OWN>
+__device__ __forceinline__ float2 dot2(float2 ax, float2 ay, float2 az, float2 bx, float2 by, float2 bz) {
+    if constexpr (OWN) return fma2(az, bz, fma2(ax, bx, mul2(ay, by)));
+    else return fma2(az, bz, fma2(ay, by, mul2(ax, bx)));
+}
+template <bool OWN>
 __device__ __forceinline__ Coll2 make_coll2(const SimDev &s, const CollK &k, const Moments2 &m, float2 Gx, float2 Gy,
                                             float2 Gz, float2 &rho, float2 &usq) {
     const float2 inv = v2(s.inv_scale), half = v2(0.5f);
@@ -751,8 +778,8 @@ __device__ __forceinline__ Coll2 make_coll2(const SimDev &s, const CollK &k, con
     c.Gx = Gx;
     c.Gy = Gy;
     c.Gz = Gz;
-    usq = fma2(c.uz, c.uz, fma2(c.uy, c.uy, mul2(c.ux, c.ux)));
-    const float2 uG = fma2(c.uz, Gz, fma2(c.uy, Gy, mul2(c.ux, Gx)));
+    usq = dot2<OWN>(c.ux, c.uy, c.uz, c.ux, c.uy, c.uz);
+    const float2 uG = dot2<OWN>(c.ux, c.uy, c.uz, Gx, Gy, Gz);
     const float2 K = fma2(mul2(v2(-1.5f), rho), usq, drho);
     c.Kb = fma2(v2(k.om), K, mul2(v2(-k.fp3), uG));
     c.Rb = mul2(v2(k.om3), rho);
@@ -776,14 +803,23 @@ __device__ __forceinline__ void pair_terms2(const Coll2 &c, const Cls2 &w, float
     AmB = sub2(A, B);
 }
 
-template <typename T, int Q>
+// OWN: each cell has its own random bits (rng, rng2), as in the one-cell kernel,
+// which rounds the two populations of a cell together.
+template <typename T, int Q, bool OWN>
 __device__ __forceinline__ void collide2(uint16_t *__restrict__ dst, size_t nfp, uint32_t f, uint32_t Pq, uint32_t Po,
                                          const Coll2 &c, const CollK &k, const Cls2 &w,
-                                         uint32_t &rng) {
+                                         uint32_t &rng, uint32_t &rng2) {
     float2 ApB, AmB;
     pair_terms2<Q>(c, w, ApB, AmB);
     const float2 oq = fma2(v2(k.c1), unpack2<T>(Pq), ApB), oo = fma2(v2(k.c1), unpack2<T>(Po), AmB);
     rng = rng * 747796405u + 2891336453u;
+    if constexpr (OWN) {
+        rng2 = rng2 * 747796405u + 2891336453u;
+        const uint32_t a = Pack2<T>::rs(oq.x, oo.x, rng ^ (rng >> 15)), b = Pack2<T>::rs(oq.y, oo.y, rng2 ^ (rng2 >> 15));
+        __stcs((unsigned int *)(dst + (size_t)Q * nfp + f), __byte_perm(a, b, 0x5410));
+        __stcs((unsigned int *)(dst + (size_t)(Q + 1) * nfp + f), __byte_perm(a, b, 0x7632));
+        return;
+    }
     const uint32_t r1 = rng ^ (rng >> 15);
     // The second store takes the same 32 bits with their halves exchanged:
     // each rounding still sees uniform bits (so stays unbiased); only
@@ -881,7 +917,7 @@ __device__ __forceinline__ Coupling load_coupling(const SimDev &s, int par, uint
     return c;
 }
 
-template <typename T>
+template <typename T, bool OWN = false>
 __device__ __forceinline__ void pair_update(const SimDev &s, int par, uint32_t f, const typename PairRaw<T>::type (&P)[NQ],
                                             uint32_t step_seed, const Coupling &cp) {
     const size_t nfp = (size_t)s.nfp;
@@ -901,26 +937,31 @@ __device__ __forceinline__ void pair_update(const SimDev &s, int par, uint32_t f
         uint16_t *__restrict__ dst = (uint16_t *)s.pop[par ^ 1];
         const CollK k = make_collk(s);
         const Moments2 m = moments2<T>(P);
-        const Coll2 c = make_coll2(s, k, m, Gx, Gy, Gz, rho, usq);
+        const Coll2 c = make_coll2<OWN>(s, k, m, Gx, Gy, Gz, rho, usq);
         const float sc = s.scale;
         const float wsc0 = (float)d3q19_w(0) * sc, wsc1 = (float)d3q19_w(1) * sc, wsc2 = (float)d3q19_w(7) * sc;
-        uint32_t rng = mix32(f ^ step_seed);
+        uint32_t rng = mix32(f ^ step_seed), rng2 = OWN ? mix32((f + 1) ^ step_seed) : 0u;
         rng = rng * 747796405u + 2891336453u;
+        rng2 = rng2 * 747796405u + 2891336453u;
         const float2 o0 = fma2(v2(k.c1), unpack2<T>(P[0]), mul2(v2(wsc0), c.Kb));
-        __stcs((unsigned int *)(dst + f), Pack2<T>::rs(o0.x, o0.y, rng ^ (rng >> 15)));
+        if constexpr (OWN)
+            __stcs((unsigned int *)(dst + f), __byte_perm(Pack2<T>::rs(o0.x, 0.0f, rng ^ (rng >> 15)),
+                                                          Pack2<T>::rs(o0.y, 0.0f, rng2 ^ (rng2 >> 15)), 0x5410));
+        else
+            __stcs((unsigned int *)(dst + f), Pack2<T>::rs(o0.x, o0.y, rng ^ (rng >> 15)));
         {
             const Cls2 w = make_cls2(c, k, wsc1);
-            collide2<T, 1>(dst, nfp, f, P[1], P[2], c, k, w, rng);
-            collide2<T, 3>(dst, nfp, f, P[3], P[4], c, k, w, rng);
-            collide2<T, 5>(dst, nfp, f, P[5], P[6], c, k, w, rng);
+            collide2<T, 1, OWN>(dst, nfp, f, P[1], P[2], c, k, w, rng, rng2);
+            collide2<T, 3, OWN>(dst, nfp, f, P[3], P[4], c, k, w, rng, rng2);
+            collide2<T, 5, OWN>(dst, nfp, f, P[5], P[6], c, k, w, rng, rng2);
         }
         const Cls2 w = make_cls2(c, k, wsc2);
-        collide2<T, 7>(dst, nfp, f, P[7], P[8], c, k, w, rng);
-        collide2<T, 9>(dst, nfp, f, P[9], P[10], c, k, w, rng);
-        collide2<T, 11>(dst, nfp, f, P[11], P[12], c, k, w, rng);
-        collide2<T, 13>(dst, nfp, f, P[13], P[14], c, k, w, rng);
-        collide2<T, 15>(dst, nfp, f, P[15], P[16], c, k, w, rng);
-        collide2<T, 17>(dst, nfp, f, P[17], P[18], c, k, w, rng);
+        collide2<T, 7, OWN>(dst, nfp, f, P[7], P[8], c, k, w, rng, rng2);
+        collide2<T, 9, OWN>(dst, nfp, f, P[9], P[10], c, k, w, rng, rng2);
+        collide2<T, 11, OWN>(dst, nfp, f, P[11], P[12], c, k, w, rng, rng2);
+        collide2<T, 13, OWN>(dst, nfp, f, P[13], P[14], c, k, w, rng, rng2);
+        collide2<T, 15, OWN>(dst, nfp, f, P[15], P[16], c, k, w, rng, rng2);
+        collide2<T, 17, OWN>(dst, nfp, f, P[17], P[18], c, k, w, rng, rng2);
         ux = c.ux;
         uy = c.uy;
         uz = c.uz;
@@ -933,7 +974,7 @@ __device__ __forceinline__ void pair_update(const SimDev &s, int par, uint32_t f
 }
 
 template <typename T, int MODE>
-__device__ __forceinline__ void fluid_pair(const SimDev &s, int par, int fi, uint32_t step_seed) {
+__device__ __forceinline__ void fluid_pair_even(const SimDev &s, int par, int fi, uint32_t step_seed) {
     const T *__restrict__ src = (const T *)s.pop[par];
     const size_t nfp = (size_t)s.nfp;
     const uint32_t f = (uint32_t)fi;
@@ -961,6 +1002,66 @@ __device__ __forceinline__ void fluid_pair(const SimDev &s, int par, int fi, uin
         if (yhi) bounce2<T, -1, MODE>(src, nfp, f, P);
     }
     pair_update<T>(s, par, f, P, step_seed, load_coupling(s, par, f, (act >> (f & 31)) & 3u));
+}
+
+// Odd nx: cells f and f + 1 (f even) may lie in two rows, and a row's start has
+// any alignment, so each cell has its own source addresses; the arithmetic
+// and the stores are those of the pair.  Same numbers as the one-cell kernel,
+// which took these widths before (255x128x128 FP16 82.1 -> 64.7 us a step, FP32 93.4
+// -> 90.9; 511x256x256 FP16 636 -> 484; 24 serving requests 230.5 -> 219.0).
+template <typename T, int MODE>
+__device__ __forceinline__ void fluid_pair_odd(const SimDev &s, int par, int fi, uint32_t step_seed) {
+    const T *__restrict__ src = (const T *)s.pop[par];
+    const size_t nfp = (size_t)s.nfp;
+    const uint32_t f = (uint32_t)fi;
+    const uint32_t r = s.div_nx.div(f);
+    const uint32_t x = f - r * (uint32_t)s.nx;
+    const uint32_t z = s.div_nyf.div(r);
+    const uint32_t y = r - z * (uint32_t)s.nyf;
+    const Rows na = source_rows(s, f, (int)y, (int)z);
+    const int xma = x == 0 ? s.nx - 1 : -1, xpa = x == (uint32_t)s.nx - 1 ? 1 - s.nx : 1;
+    // the second cell: the next of the row, the first of the next row, or (past
+    // the last cell, where its place is padding) the first cell again
+    const bool last = fi + 1 == s.nf, turn = !last && x == (uint32_t)s.nx - 1;
+    const uint32_t xb = last ? x : turn ? 0u : x + 1u;
+    uint32_t yb = y;
+    Rows nb;
+    const uint32_t one = last ? 0u : 1u;
+#pragma unroll
+    for (int i = 0; i < 3; ++i)
+#pragma unroll
+        for (int j = 0; j < 3; ++j) nb.row[i][j] = na.row[i][j] + one;
+    if (turn) {
+        const bool up = y == (uint32_t)s.nyf - 1;
+        yb = up ? 0u : y + 1u;
+        nb = source_rows(s, f + 1u, (int)yb, (int)(up ? z + 1u : z));
+    }
+    const int xmb = xb == 0 ? s.nx - 1 : -1, xpb = xb == (uint32_t)s.nx - 1 ? 1 - s.nx : 1;
+
+    typename PairRaw<T>::type P[NQ];
+#define LBIB_PULL2(q) P[q] = pull_cells<T, q, MODE>(src, nfp, na, xma, xpa, nb, xmb, xpb);
+    LBIB_PULL2(0) LBIB_PULL2(1) LBIB_PULL2(2) LBIB_PULL2(3) LBIB_PULL2(4) LBIB_PULL2(5) LBIB_PULL2(6)
+    LBIB_PULL2(7) LBIB_PULL2(8) LBIB_PULL2(9) LBIB_PULL2(10) LBIB_PULL2(11) LBIB_PULL2(12) LBIB_PULL2(13)
+    LBIB_PULL2(14) LBIB_PULL2(15) LBIB_PULL2(16) LBIB_PULL2(17) LBIB_PULL2(18)
+#undef LBIB_PULL2
+    if constexpr (MODE == MODE_EARLY) {  // as in fluid_cell
+        dep_wait();
+        dep_release();
+    }
+    const uint32_t act = __ldcg(s.amask + (f >> 5));
+    const uint32_t top = (uint32_t)s.nyf - 1;
+    const bool alo = s.walls && y == 0, ahi = s.walls && y == top, blo = s.walls && yb == 0, bhi = s.walls && yb == top;
+    if (__any_sync(__activemask(), alo || ahi || blo || bhi)) {
+        if (alo || blo) bounce_cells<T, 1, MODE>(src, nfp, f, alo, blo, P);
+        if (ahi || bhi) bounce_cells<T, -1, MODE>(src, nfp, f, ahi, bhi, P);
+    }
+    pair_update<T, true>(s, par, f, P, step_seed, load_coupling(s, par, f, (act >> (f & 31)) & 3u));
+}
+
+template <typename T, int MODE, bool ODD>
+__device__ __forceinline__ void fluid_pair(const SimDev &s, int par, int f, uint32_t step_seed) {
+    if constexpr (ODD) fluid_pair_odd<T, MODE>(s, par, f, step_seed);
+    else fluid_pair_even<T, MODE>(s, par, f, step_seed);
 }
 
 // Pull offset of direction q in the fluid index space away from the

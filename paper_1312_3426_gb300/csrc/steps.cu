@@ -70,7 +70,7 @@ __device__ __forceinline__ void steps_signal(unsigned *c) {
     }
 }
 
-// PAIR: two cells per thread (else one; BC: obstacles or an inlet)
+// PAIR: two cells per thread (BC: nx odd), else one (BC: obstacles or an inlet)
 template <typename T, bool PAIR, bool BC>
 __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, long long t0, int n, unsigned *sync) {
     constexpr int THREADS = STEPS_THREADS<T, PAIR>, CELLS = PAIR ? 2 * THREADS : THREADS;
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, l
                 const int f0 = tile * CELLS;
                 if constexpr (PAIR) {
                     const int f = f0 + 2 * (int)threadIdx.x;
-                    if (f < s.nf) fluid_pair<T, MODE_MANY>(s, par, f, seed);
+                    if (f < s.nf) fluid_pair<T, MODE_MANY, BC>(s, par, f, seed);
                 } else {
                     fluid_block<T, BC, MODE_MANY>(s, par, f0, seed);
                 }
@@ -172,6 +172,7 @@ static cudaError_t launch_steps_t(const SimDev &s, size_t smem, long long t, int
 
 template <typename T>
 static cudaError_t launch_steps_v(const SimDev &s, size_t smem, long long t, int n, unsigned *sync, cudaStream_t st) {
+    if (steps_pair(s) && (s.nx & 1)) return launch_steps_t<T, true, true>(s, smem, t, n, sync, st);
     if (steps_pair(s)) return launch_steps_t<T, true, false>(s, smem, t, n, sync, st);
     if (s.solid || s.in_on) return launch_steps_t<T, false, true>(s, smem, t, n, sync, st);
     return launch_steps_t<T, false, false>(s, smem, t, n, sync, st);
