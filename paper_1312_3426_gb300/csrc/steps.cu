@@ -11,7 +11,9 @@
 //                  nodes take 7 us, at about one sector a cycle);
 //   [barrier]
 //   then, by role  the first blocks: the membrane forces of one object each, for
-//                  the next step; the others: the fluid cells, in tiles;
+//                  the next step (and, with repulsion between objects, a
+//                  barrier over these blocks and the repulsion on its nodes);
+//                  the others: the fluid cells, a warp's 32 or 64 at a time;
 //   [barrier]
 // The barriers are counters in global memory that only grow (reset before the
 // launch), added to after a block barrier and a fence, read with acquire by
@@ -73,11 +75,11 @@ __device__ __forceinline__ void steps_signal(unsigned *c) {
 // PAIR: two cells per thread (BC: nx odd), else one (BC: obstacles or an inlet)
 template <typename T, bool PAIR, bool BC>
 __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, long long t0, int n, unsigned *sync) {
-    constexpr int THREADS = STEPS_THREADS<T, PAIR>, CELLS = PAIR ? 2 * THREADS : THREADS;
+    constexpr int THREADS = STEPS_THREADS<T, PAIR>;
     unsigned *nodes_done = sync, *boxes_done = sync + 16, *done = sync + 32;
     const unsigned blocks = gridDim.x;
     const int nobj = s.nobj, b = (int)blockIdx.x, nfluid = (int)blocks - nobj;
-    const int tiles = (s.nf + CELLS - 1) / CELLS;
+    const int groups = (s.nf + (PAIR ? 63 : 31)) / (PAIR ? 64 : 32);
     for (int k = 0; k < n; ++k) {
         const long long t = t0 + k;
         const int par = (int)(t & 1);
@@ -98,13 +100,17 @@ __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, l
             }
         } else {
             const uint32_t seed = step_seed(t);
-            for (int tile = b - nobj; tile < tiles; tile += nfluid) {
-                const int f0 = tile * CELLS;
+            // groups of a warp's cells, one after the other to different blocks,
+            // so that in the last round every block has as many warps at work
+            constexpr int GROUP = PAIR ? 64 : 32;
+            const int lane = (int)threadIdx.x & 31;
+            for (int g = b - nobj + nfluid * (int)(threadIdx.x >> 5); g < groups; g += nfluid * (THREADS / 32)) {
                 if constexpr (PAIR) {
-                    const int f = f0 + 2 * (int)threadIdx.x;
+                    const int f = GROUP * g + 2 * lane;
                     if (f < s.nf) fluid_pair<T, MODE_MANY, BC>(s, par, f, seed);
                 } else {
-                    fluid_block<T, BC, MODE_MANY>(s, par, f0, seed);
+                    const int f = GROUP * g + lane;
+                    if (f < s.nf) fluid_cell<T, BC, MODE_MANY>(s, par, f, active_word(s, f), seed);
                 }
             }
         }
@@ -112,15 +118,19 @@ __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, l
     }
 }
 
-// Two cells per thread where the shape allows; FP32 (the same bits either
+// Two cells per thread where the kernel allows; FP32 (the same bits either
 // way) only where one cell per thread takes more than two rounds of the
-// blocks (64x48x48 with 3 cells 12.7 against 14.6 us a step).
-static bool steps_pair(const SimDev &s) {
+// blocks (64x48x48 with 3 cells 12.1 against 13.0 us a step, without objects 101x37x53
+// 5.7 against 6.3; 128x64x64 with 20 cells 17.6 against 15.9) and the objects are not
+// so large that the step waits for their membrane blocks, which then have 512
+// threads (8 level-4 cells in 128x64x64 27.9 against 31.4).
+static bool steps_pair(const SimDev &s, int max_edges) {
     if (fluid_kernel_kind(s) == 0) return false;
-    return s.prec != LBIB_POP_F32 || s.nf > 2 * STEPS_THREADS<float, false> * (device_sms() - s.nobj);
+    return s.prec != LBIB_POP_F32 ||
+           (s.nf > 2 * STEPS_THREADS<float, false> * (device_sms() - s.nobj) && (s.nobj == 0 || max_edges <= 4096));
 }
-static int steps_tiles(const SimDev &s) {
-    const int cells = !steps_pair(s)             ? STEPS_THREADS<float, false>
+static int steps_tiles(const SimDev &s, int max_edges) {
+    const int cells = !steps_pair(s, max_edges)         ? STEPS_THREADS<float, false>
                       : s.prec == LBIB_POP_F32 ? 2 * STEPS_THREADS<float, true>
                                                : 2 * STEPS_THREADS<__half, true>;
     return (s.nf + cells - 1) / cells;
@@ -129,62 +139,69 @@ static int steps_tiles(const SimDev &s) {
 // Blocks for the fluid cells: what is left of the SMs, one tile each if that is
 // fewer.  Beside objects, whose membrane blocks take as long as two or three
 // rounds of tiles, half as many do (64x48x48 with 3 cells: 49 blocks instead of
-// 95 at 12.9 us a step), and simulations on other streams find room (8 of
+// 95 at the same time a step), and simulations on other streams find room (8 of
 // these on 8 streams 4.5 us a simulation and step against 12.8 with 95 blocks,
 // 7.9 with separate launches, which the host bounds).
-static int steps_fluid_blocks(const SimDev &s) {
-    const int sms = device_sms() - s.nobj, tiles = steps_tiles(s);
+static int steps_fluid_blocks(const SimDev &s, int max_edges) {
+    const int sms = device_sms() - s.nobj, tiles = steps_tiles(s, max_edges);
     if (s.nobj > 0 && tiles > sms / 4 && tiles <= sms) return (tiles + 1) / 2;
     return tiles < sms ? tiles : sms;
 }
 
-// Up to 8 rounds of the fluid blocks (without objects 32 tiles to 5 rounds),
-// and objects on half of the SMs at most.  us a step, one launch against
-// separate ones:
-//   sphere 40x20x20                 9.4 / 15.0
-//   no objects 101x37x53            6.4 /  8.3    128x96x96 FP16  16.5 / 18.5
-//   3 cells 64x48x48 FP16          12.9 / 22.4
-//   20 cells 117x70x66 FP32        20.3 / 25.6
-//   20 cells 128x64x64 FP32        17.2 / 24.3    FP16  15.2 / 24.2
-//   8 level-4 cells 128x64x64 FP32 30.7 / 39.3
-//   20 cells 96x96x96 FP32         31.0 / 32.9    160x96x96 FP16  32.6 / 34.3
-// beyond (10 rounds at 160x96x96 FP32, 160x128x96 FP16) they are equal.
+// Up to 8 rounds of the fluid blocks (6 of the FP32 two-cells blocks, which
+// have 16 warps; without objects 32 tiles to 5 rounds), and objects on half of
+// the SMs at most.  us a step, one launch against separate ones:
+//   sphere 40x20x20                 8.2 / 12.7
+//   no objects 101x37x53            5.7 /  6.2    128x96x96 FP16  16.7 / 18.6
+//   3 cells 64x48x48 FP16          11.5 / 20.5
+//   20 cells 117x70x66 FP32        17.0 / 22.5
+//   20 cells 128x64x64 FP32        16.0 / 22.8    FP16  12.9 / 22.1
+//   8 level-4 cells 128x64x64 FP32 28.1 / 37.7
+//   20 cells 120x80x80 FP32        25.9 / 26.6    160x96x96 FP16  29.3 / 30.9
+//   10 bodies with repulsion among posts FP16: 199x50x30 12.8 / 32.4, 200x64x64 26.0 / 33.8
+// beyond (6.4 rounds at 96x96x96 FP32 30.6 / 28.8, 9.5 at 160x128x96 FP16 37.3 /
+// 37.4) they are equal or worse.
 bool steps_fit(const SimDev &s, int max_nodes, int max_edges) {
     const int sms = device_sms();
     if ((s.rep_on && s.nobj > REPEL_MAX_OBJECTS) || (s.nobj > 0 && ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX)) return false;
-    const int tiles = steps_tiles(s);
+    const int tiles = steps_tiles(s, max_edges);
     if (s.nobj == 0) return tiles >= 32 && tiles <= 5 * sms;
-    return 2 * s.nobj <= sms && tiles <= 8 * (sms - s.nobj);
+    const int rounds = s.prec == LBIB_POP_F32 && steps_pair(s, max_edges) ? 6 : 8;
+    return 2 * s.nobj <= sms && tiles <= rounds * (sms - s.nobj);
 }
 
 template <typename T, bool PAIR, bool BC>
-static cudaError_t launch_steps_t(const SimDev &s, size_t smem, long long t, int n, unsigned *sync, cudaStream_t st) {
+static cudaError_t launch_steps_t(const SimDev &s, size_t smem, int fluid, long long t, int n, unsigned *sync,
+                                  cudaStream_t st) {
     static SmemAttr attr;
     void *fn = (void *)k_steps<T, PAIR, BC>;
     cudaError_t e = attr.ensure(fn, smem, false);
     if (e == cudaSuccess) e = cudaMemsetAsync(sync, 0, 192, st);
     if (e != cudaSuccess) return e;
-    const int fluid = steps_fluid_blocks(s);
     SimDev d = s;
     void *args[] = {&d, &t, &n, &sync};
     return cudaLaunchCooperativeKernel(fn, dim3((unsigned)(s.nobj + fluid)), dim3(STEPS_THREADS<T, PAIR>), args, smem, st);
 }
 
 template <typename T>
-static cudaError_t launch_steps_v(const SimDev &s, size_t smem, long long t, int n, unsigned *sync, cudaStream_t st) {
-    if (steps_pair(s) && (s.nx & 1)) return launch_steps_t<T, true, true>(s, smem, t, n, sync, st);
-    if (steps_pair(s)) return launch_steps_t<T, true, false>(s, smem, t, n, sync, st);
-    if (s.solid || s.in_on) return launch_steps_t<T, false, true>(s, smem, t, n, sync, st);
-    return launch_steps_t<T, false, false>(s, smem, t, n, sync, st);
+static cudaError_t launch_steps_v(const SimDev &s, int max_nodes, int max_edges, long long t, int n, unsigned *sync,
+                                  cudaStream_t st) {
+    const size_t smem = s.nobj > 0 ? ib_smem_bytes(max_nodes, max_edges) : 0;
+    const int fluid = steps_fluid_blocks(s, max_edges);
+    if (steps_pair(s, max_edges)) {
+        if (s.nx & 1) return launch_steps_t<T, true, true>(s, smem, fluid, t, n, sync, st);
+        return launch_steps_t<T, true, false>(s, smem, fluid, t, n, sync, st);
+    }
+    if (s.solid || s.in_on) return launch_steps_t<T, false, true>(s, smem, fluid, t, n, sync, st);
+    return launch_steps_t<T, false, false>(s, smem, fluid, t, n, sync, st);
 }
 
 cudaError_t launch_steps(const SimDev &s, int max_nodes, int max_edges, long long t, int n, unsigned *sync,
                          cudaStream_t st) {
-    const size_t smem = s.nobj > 0 ? ib_smem_bytes(max_nodes, max_edges) : 0;
     switch (s.prec) {
-        case LBIB_POP_F32: return launch_steps_v<float>(s, smem, t, n, sync, st);
-        case LBIB_POP_F16S: return launch_steps_v<__half>(s, smem, t, n, sync, st);
-        default: return launch_steps_v<__nv_bfloat16>(s, smem, t, n, sync, st);
+        case LBIB_POP_F32: return launch_steps_v<float>(s, max_nodes, max_edges, t, n, sync, st);
+        case LBIB_POP_F16S: return launch_steps_v<__half>(s, max_nodes, max_edges, t, n, sync, st);
+        default: return launch_steps_v<__nv_bfloat16>(s, max_nodes, max_edges, t, n, sync, st);
     }
 }
 
