@@ -935,11 +935,14 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
         if (r != LBIB_OK) return r;
         LBIB_CUDA(s, cudaEventRecord(ev[0], st), "profile event");
     }
-    const int threads = s->membrane_auto && s->cluster == 1
-                            ? membrane_threads((int)s->objs.size(), s->max_edges,
-                                               s->overlap ? fluid_time_us(s->d.nf, s->p.precision) : 0.0)
-                            : s->membrane_threads;
-    LBIB_CUDA(s, launch_membrane(s->d, s->max_nodes, s->max_edges, s->cluster, s->membrane_clusters, threads,
+    int threads = s->membrane_threads, clusters = s->membrane_clusters;
+    if (s->membrane_auto && s->cluster == 1) {
+        const int nobj = (int)s->objs.size();
+        const double fluid_us = s->overlap ? fluid_time_us(s->d.nf, s->p.precision) : 0.0;
+        threads = membrane_threads(nobj, s->max_edges, fluid_us);
+        if (clusters == 0) membrane_share(nobj, s->max_nodes, s->max_edges, fluid_us, clusters, threads);
+    }
+    LBIB_CUDA(s, launch_membrane(s->d, s->max_nodes, s->max_edges, s->cluster, clusters, threads,
                                  s->membrane_group, st), "membrane forces");
     LBIB_CUDA(s, launch_repulsion(s->d, s->max_nodes, st), "repulsion");
     if (ev) LBIB_CUDA(s, cudaEventRecord(ev[1], st), "profile event");

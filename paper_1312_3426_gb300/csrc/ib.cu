@@ -68,6 +68,33 @@ int membrane_threads(int nobj, int max_edges, double fluid_us) {
     return best;
 }
 
+// Where the objects come in several rounds, one block on each SM goes from object
+// to object beside the fluid update: sets the block count and threads of such a
+// launch.  One block per object has blocks waiting for room all the time, and
+// while blocks of the higher priority wait, no fluid block starts.  The fewest
+// threads that let the rounds end within 85% of the fluid update (half of it
+// for two rounds, of which the second may be all but empty); elsewhere one block
+// per object is as good.  us a step, this against one each: 2000 level-3 cells
+// 512x256x256 FP32 894 / 932 (BF16 645 / 645), 420 767 / 777, 500 in 512x128x128 229.5 /
+// 236.5; level 4, whose blocks fill an SM's shared memory: 300 in 512x256x256 FP32
+// 789 / 879, BF16 526 / 602, 700 FP32 866 / 1077, BF16 654 / 799.  (200 level-3 cells in
+// 256x128x128 with 152 blocks of 768 threads: 121 / 113.)
+bool membrane_share(int nobj, int max_nodes, int max_edges, double fluid_us, int &blocks, int &threads) {
+    const int sms = device_sms(), rounds = (nobj + sms - 1) / sms;
+    if (rounds < 2) return false;
+    // blocks that leave no room for a second one may as well be wide
+    const bool alone = 2 * ib_smem_bytes(max_nodes, membrane_in_global(max_nodes, max_edges, 1) ? 0 : max_edges) > IB_SMEM_MAX;
+    for (int t : {192, 256, 384, 512, 768}) {
+        if (t > 384 && !alone) break;
+        const double us = 10.0 + rounds * (10.0 + 3.5 * ((max_edges + t - 1) / t));
+        if (us > (rounds > 2 ? 0.85 : 0.5) * fluid_us) continue;
+        blocks = sms;
+        threads = t;
+        return true;
+    }
+    return false;
+}
+
 cudaError_t launch_membrane(const SimDev &s, int max_nodes, int max_edges, int cluster, int max_clusters, int threads,
                             int group, cudaStream_t st) {
     if (s.nobj == 0) return cudaSuccess;

@@ -312,6 +312,8 @@ size_t membrane_scalar_bytes(int max_edges);  // per object
 // Threads per object of a membrane launch of nobj objects (one per block)
 // beside a fluid update of fluid_us microseconds (0: nothing beside it).
 int membrane_threads(int nobj, int max_edges, double fluid_us);
+// Whether fewer blocks than objects go through them, with how many blocks and threads.
+bool membrane_share(int nobj, int max_nodes, int max_edges, double fluid_us, int &blocks, int &threads);
 // Time of the fluid update of nf cells: its populations in and out at 6 TB/s.
 inline double fluid_time_us(int64_t nf, int prec) { return (double)nf * 38 * (prec == LBIB_POP_F32 ? 4 : 2) / 6.0e6; }
 // SM count of the current device (cached per device)
