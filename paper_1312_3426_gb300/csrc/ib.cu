@@ -1,5 +1,5 @@
 // Immersed-boundary kernels of one simulation: the membrane part (one
-// thread-block cluster per object) and the coupling part (one thread per
+// thread-block cluster per object) and the coupling part (two threads per
 // node), as described in ib_core.cuh.
 #include "ib_core.cuh"
 

@@ -118,8 +118,8 @@ lbib_status sim_edge_scratch(lbib_sim *s);
 cudaError_t sim_remark(lbib_sim *s, cudaStream_t st);
 // Nodes per block of the node kernel: 64 while the knob has its default.  A node waits for two
 // rounds of memory, one after the other, and small blocks leave and refill an
-// SM one by one (steps with 64 against 256: 3 cells 64x48x48 21.8 / 22.6 us,
-// 20 cells 117x70x66 26.4 / 27.3, 200 cells 256x128x128 FP32 126.9 / 128.1,
-// the batch of 24 serving requests 293 / 295).
+// SM one by one (steps with 32 / 64 / 128: 200 cells 256x128x128 FP16 82.9 / 83.1 /
+// 83.3 us, 2000 cells FP32 934 / 934 / 937, 24 serving requests 229.9 / 230.6 /
+// 231.8; 256 was slower still).
 inline int node_chunk(const lbib_sim *s) { return s->node_auto ? 64 : s->node_threads; }
 }  // namespace lbib
