@@ -676,13 +676,10 @@ lbib_status lbib_template_create(lbib_sim *s, int tid, const double *xyz, int nn
     md.Sg0 = T.Sg0;
     md.V0 = T.V0;
     s->tpl_mem_dev.push_back(md);
-    const int ne = T.ne;
     s->topo.push_back(std::move(T));
     s->tpl_dev.push_back(dv);
     s->tpl_mem.push_back(mem);
     s->tpl_bytes += bytes;
-    s->max_nodes = std::max(s->max_nodes, nn);
-    s->max_edges = std::max(s->max_edges, ne);
     s->tables_dirty = true;
     return LBIB_OK;
 }
@@ -772,6 +769,8 @@ lbib_status lbib_object_add(lbib_sim *s, int oid, int tid, const double origin[3
     s->fext.insert(s->fext.end(), {0.f, 0.f, 0.f});
 
     s->nn_total += T.nn;
+    s->max_nodes = std::max(s->max_nodes, T.nn);
+    s->max_edges = std::max(s->max_edges, T.ne);
     s->host_newer = true;
     s->tables_dirty = true;
     return LBIB_OK;

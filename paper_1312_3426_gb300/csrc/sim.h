@@ -28,7 +28,7 @@ struct lbib_sim {
     std::vector<lbib::MemDev> tpl_mem_dev;  // membrane records of the templates (first: per object)
     std::vector<void *> tpl_mem;        // device records of every template
     size_t tpl_bytes = 0;
-    int max_nodes = 0;                  // largest template
+    int max_nodes = 0;                  // of the largest object (templates may have none)
     int max_edges = 0;
     size_t edge_bytes = 0;              // of SimDev::edge_scal
 
