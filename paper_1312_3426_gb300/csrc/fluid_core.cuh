@@ -652,15 +652,16 @@ __device__ __forceinline__ typename PairRaw<T>::type pull_cells(const T *__restr
                                                                 int xma, int xpa, const Rows &nb, int xmb, int xpb) {
     return PairRaw<T>::template ld<MODE>(src + (size_t)Q * nfp, source_cell<Q>(na, xma, xpa), source_cell<Q>(nb, xmb, xpb));
 }
+// last: the pair's second place is padding (see fluid_pair_odd) and takes the first cell's value
 template <typename T, int EY, int MODE>
-__device__ __forceinline__ void bounce_cells(const T *__restrict__ src, size_t nfp, uint32_t f, bool a, bool b,
+__device__ __forceinline__ void bounce_cells(const T *__restrict__ src, size_t nfp, uint32_t f, bool a, bool b, bool last,
                                              typename PairRaw<T>::type (&P)[NQ]) {
 #pragma unroll
     for (int q = 1; q < NQ; ++q)
         if (d3q19_ey(q) == EY) {
             const auto own = PairRaw<T>::template ld<MODE>(src + (size_t)d3q19_opp(q) * nfp, f);
-            if constexpr (sizeof(T) == 4) P[q] = make_float2(a ? own.x : P[q].x, b ? own.y : P[q].y);
-            else P[q] = __byte_perm(P[q], own, (a ? 0x0054u : 0x0010u) | (b ? 0x7600u : 0x3200u));
+            if constexpr (sizeof(T) == 4) P[q] = make_float2(a ? own.x : P[q].x, b ? (last ? own.x : own.y) : P[q].y);
+            else P[q] = __byte_perm(P[q], own, (a ? 0x0054u : 0x0010u) | (b ? (last ? 0x5400u : 0x7600u) : 0x3200u));
         }
 }
 
@@ -1021,7 +1022,8 @@ __device__ __forceinline__ void fluid_pair_odd(const SimDev &s, int par, int fi,
     const Rows na = source_rows(s, f, (int)y, (int)z);
     const int xma = x == 0 ? s.nx - 1 : -1, xpa = x == (uint32_t)s.nx - 1 ? 1 - s.nx : 1;
     // the second cell: the next of the row, the first of the next row, or (past
-    // the last cell, where its place is padding) the first cell again
+    // the last cell) the first cell again: its place is padding, which any
+    // read-out may have written to, so what it holds does not count
     const bool last = fi + 1 == s.nf, turn = !last && x == (uint32_t)s.nx - 1;
     const uint32_t xb = last ? x : turn ? 0u : x + 1u;
     uint32_t yb = y;
@@ -1052,10 +1054,12 @@ __device__ __forceinline__ void fluid_pair_odd(const SimDev &s, int par, int fi,
     const uint32_t top = (uint32_t)s.nyf - 1;
     const bool alo = s.walls && y == 0, ahi = s.walls && y == top, blo = s.walls && yb == 0, bhi = s.walls && yb == top;
     if (__any_sync(__activemask(), alo || ahi || blo || bhi)) {
-        if (alo || blo) bounce_cells<T, 1, MODE>(src, nfp, f, alo, blo, P);
-        if (ahi || bhi) bounce_cells<T, -1, MODE>(src, nfp, f, ahi, bhi, P);
+        if (alo || blo) bounce_cells<T, 1, MODE>(src, nfp, f, alo, blo, last, P);
+        if (ahi || bhi) bounce_cells<T, -1, MODE>(src, nfp, f, ahi, bhi, last, P);
     }
-    pair_update<T, true>(s, par, f, P, step_seed, load_coupling(s, par, f, (act >> (f & 31)) & 3u));
+    Coupling cp = load_coupling(s, par, f, (act >> (f & 31)) & 3u);
+    if (last) cp.b = cp.a;
+    pair_update<T, true>(s, par, f, P, step_seed, cp);
 }
 
 template <typename T, int MODE, bool ODD>
