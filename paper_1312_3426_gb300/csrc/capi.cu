@@ -3,8 +3,6 @@
 // sticky error model.  Host code only; the kernels live in fluid.cu, ib.cu
 // and batch.cu.
 #include <cuda_runtime.h>
-#include <sys/mman.h>
-#include <unistd.h>
 
 #include <algorithm>
 #include <atomic>
@@ -13,11 +11,11 @@
 #include <cstring>
 #include <initializer_list>
 #include <string>
-#include <thread>
 #include <vector>
 
 #include "lbib.h"
 #include "lbib_internal.h"
+#include "prefault.h"
 #include "sim.h"
 #include "topology.h"
 
@@ -144,39 +142,6 @@ static void *transfer_scratch(lbib_sim *s, size_t bytes) {
     if (s->solid_mem || bytes > (size_t)NQ * s->d.nfp * pop_elem_bytes(s->p.precision)) return nullptr;
     return s->d.pop[(s->t + 1) & 1];
 }
-
-// Faults the pages of a large read-out's destination in beside the wait for
-// the device: a fresh array costs more in page faults than the copy takes
-// (400 MB: 16.5 ms with the copy, 3.6 without).  Contents stay, only whole pages
-// inside the range are touched, and where it is refused the copy faults.
-class Prefault {
-   public:
-    Prefault(void *p, size_t bytes) {
-        if (!p || bytes < MIN_BYTES) return;
-        const size_t page = (size_t)sysconf(_SC_PAGESIZE), a = align_up((size_t)p, page);
-        const size_t e = ((size_t)p + bytes) / page * page;
-        if (e <= a) return;
-        const size_t part = align_up((e - a + THREADS - 1) / THREADS, page);
-        for (int i = 0; i < THREADS && a + i * part < e; ++i) {
-            const size_t lo = a + i * part, n = std::min(part, e - lo);
-            try {
-                th_[i] = std::thread([lo, n] { madvise((void *)lo, n, 23 /* MADV_POPULATE_WRITE */); });
-            } catch (const std::exception &) {
-                return;  // no thread to be had
-            }
-        }
-    }
-    ~Prefault() { join(); }
-    void join() {
-        for (std::thread &t : th_)
-            if (t.joinable()) t.join();
-    }
-
-   private:
-    static constexpr size_t MIN_BYTES = 8 << 20;
-    static constexpr int THREADS = 4;
-    std::thread th_[THREADS];
-};
 
 // Node states from which the conversion between the FP64 host layout and the
 // FP32 pairs runs on the device (host loops take 5 ns a node and back, a
