@@ -391,11 +391,11 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * clusters of the membrane-force kernel, each looping over the objects
  * (0, default: one cluster per object; a small grid leaves most SMs to the
  * fluid kernel running beside it).  LBIB_TUNE_MEMBRANE_THREADS: threads per
- * block of the membrane-force kernel (a multiple of 32 in [32, 256];
- * default 192: with that, one object per block and cluster size 1 the step
+ * block of the membrane-force kernel (a multiple of 32 in [32, 256], or 0,
+ * the default: with one object per block and cluster size 1 the step
  * picks 128 to 1024 by the number and size of the objects and the length of
- * the fluid update beside them; fewer threads leave more of each SM to the
- * fluid kernel).  LBIB_TUNE_FLUID_KERNEL (16-bit storage): 0
+ * the fluid update beside them, else 192; fewer threads leave more of each SM
+ * to the fluid kernel).  LBIB_TUNE_FLUID_KERNEL (16-bit storage): 0
  * (default) and 1 the two-cells-per-thread kernel (where
  * there are no obstacles or inlet), 2 the warp-specialised two-cells kernel
  * (a producer warp streams the populations through shared memory with bulk
@@ -404,8 +404,8 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * slower than value 1 on a GB300, kept for comparison; lbib_batch_step runs
  * value 1 instead), 3 one cell per thread; FP32 storage ignores it.
  * LBIB_TUNE_NODE_THREADS: nodes per block of the node-update kernel (32,
- * 64, 128 or 256; with the default, 256, the step takes 64;
- * lbib_batch_step takes the first simulation's).  LBIB_TUNE_MEMBRANE_GROUP: objects per block of the
+ * 64, the default, 128 or 256; lbib_batch_step takes the first
+ * simulation's).  LBIB_TUNE_MEMBRANE_GROUP: objects per block of the
  * membrane-force kernel (1..15, default 1); above 1 each object gets
  * LBIB_TUNE_MEMBRANE_THREADS threads of a block of group x threads threads
  * (at most 1024) and the cluster knobs do not apply; the step takes as

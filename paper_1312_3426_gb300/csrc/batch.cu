@@ -120,7 +120,7 @@ struct BatchPlan {
     std::vector<uint64_t> serial;  // identity of each simulation (addresses can be reused)
     std::vector<int> nobj, nn, group;  // group: fluid kernel variant (2 * precision + BC)
     std::vector<SimDev> dev;  // descriptors the device copy holds
-    int cluster = 0, device = -1, mthreads = IB_THREADS, nthreads = IB_THREADS_DEFAULT, mgroup = 1;
+    int cluster = 0, device = -1, mthreads = IB_THREADS, nthreads = NODE_CHUNK_DEFAULT, mgroup = 1;
     SimDev *d_sims = nullptr;
     long long *d_t = nullptr;
     int2 *d_items = nullptr;  // fluid (by storage type x obstacles), then node, then membrane items
@@ -131,10 +131,9 @@ struct BatchPlan {
     // within a factor 2 of the largest, and the rest, whose largest has
     // rest_nodes nodes and rest_edges edges (0: one class)
     int n_big = 0, rest_nodes = 0, rest_edges = 0;
-    // threads per object of the two classes where that and the group have
-    // their defaults
+    // threads per object of the two classes by the rule, and whether it holds
     int big_threads = 0, rest_threads = 0;
-    bool mauto = false;
+    bool mrule = false;
     int pf_cell = 0, pf_pair = 0;  // L2 prefetch distances of the fluid launches (work items)
     cudaStream_t aux = nullptr;   // membrane kernel
     cudaStream_t aux2 = nullptr;  // membrane kernel of the smaller size class
@@ -181,7 +180,7 @@ static int fluid_group(const lbib_sim *s) {
 
 static bool plan_matches(lbib_sim *const *sims, int n, int cluster) {
     if ((int)g_plan.sims.size() != n || g_plan.cluster != cluster || g_plan.device != sims[0]->device ||
-        g_plan.nthreads != node_chunk(sims[0]))
+        g_plan.nthreads != sims[0]->node_threads)
         return false;
     for (int i = 0; i < n; ++i)
         if (g_plan.sims[i] != sims[i] || g_plan.serial[i] != sims[i]->serial ||
@@ -193,7 +192,7 @@ static bool plan_matches(lbib_sim *const *sims, int n, int cluster) {
 
 static cudaError_t build_plan(lbib_sim *const *sims, int n, int cluster, cudaStream_t st) {
     g_plan.release();
-    const int nthreads = node_chunk(sims[0]);  // of the batch
+    const int nthreads = sims[0]->node_threads;  // of the batch
     if (!g_plan.aux) {
         int lo = 0, hi = 0;
         cudaError_t e = cudaDeviceGetStreamPriorityRange(&lo, &hi);
@@ -319,7 +318,7 @@ static cudaError_t launch_membrane_batch(cudaStream_t st) {
     if (g_plan.n_mb == 0) return cudaSuccess;
     const int G = g_plan.mgroup;
     const size_t per = ib_smem_bytes(g_plan.max_nodes, g_plan.max_edges);
-    const bool own = g_plan.mauto && g_plan.cluster == 1;
+    const bool own = g_plan.mrule && g_plan.cluster == 1;
     const int T1 = own ? g_plan.big_threads : g_plan.mthreads, T2 = own ? g_plan.rest_threads : g_plan.mthreads;
     if ((G > 1 || own) && g_plan.n_big < g_plan.n_mb && per <= IB_SMEM_MAX) {
         cudaError_t e;
@@ -473,11 +472,11 @@ extern "C" lbib_status lbib_batch_step(lbib_sim *const *sims, int n, int n_steps
             if (r != LBIB_OK) return r;
         }
     if (!plan_matches(sims, n, cluster)) e = build_plan(sims, n, cluster, st);
-    if (g_plan.mthreads != sims[0]->membrane_threads || g_plan.mgroup != sims[0]->membrane_group ||
-        g_plan.mauto != sims[0]->membrane_auto) {
-        g_plan.mthreads = sims[0]->membrane_threads;  // captured in the graph
+    if (g_plan.mthreads != membrane_block(sims[0]) || g_plan.mgroup != sims[0]->membrane_group ||
+        g_plan.mrule != membrane_by_rule(sims[0])) {
+        g_plan.mthreads = membrane_block(sims[0]);  // captured in the graph
         g_plan.mgroup = sims[0]->membrane_group;
-        g_plan.mauto = sims[0]->membrane_auto;
+        g_plan.mrule = membrane_by_rule(sims[0]);
         g_plan.release_graph();
     }
     // descriptors (node arrays may have been reallocated, tables uploaded)

@@ -899,8 +899,8 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
         if (r != LBIB_OK) return r;
         LBIB_CUDA(s, cudaEventRecord(ev[0], st), "profile event");
     }
-    int threads = s->membrane_threads, clusters = s->membrane_clusters;
-    if (s->membrane_auto && s->cluster == 1) {
+    int threads = membrane_block(s), clusters = s->membrane_clusters;
+    if (membrane_by_rule(s) && s->cluster == 1) {
         const int nobj = (int)s->objs.size();
         const double fluid_us = s->overlap ? fluid_time_us(s->d.nf, s->p.precision) : 0.0;
         threads = membrane_threads(nobj, s->max_edges, fluid_us);
@@ -924,8 +924,8 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
 // Whether lbib_step runs its steps in one launch (steps.cu): a small simulation
 // whose launch knobs have their defaults, while no step is sampled.
 static bool many_steps(const lbib_sim *s) {
-    return s->overlap && s->membrane_auto && s->cluster == 1 && s->membrane_clusters == 0 && !s->early_launch &&
-           s->node_auto && !s->prof_on && !s->many_refused && s->d.fkern != 2 && steps_fit(s->d, s->max_nodes, s->max_edges);
+    return s->overlap && membrane_by_rule(s) && s->cluster == 1 && s->membrane_clusters == 0 && !s->early_launch &&
+           s->node_threads == NODE_CHUNK_DEFAULT && !s->prof_on && !s->many_refused && s->d.fkern != 2 && steps_fit(s->d, s->max_nodes, s->max_edges);
 }
 
 lbib_status lbib_step(lbib_sim *s, int n) {
@@ -991,7 +991,7 @@ lbib_status lbib_step(lbib_sim *s, int n) {
         // node kernel releases only after it) before it waits for the mask
         // and the coupling buffer.
         const bool early = s->early_launch && i > 0 && !s->prof_now;
-        if (objects) LBIB_CUDA(s, launch_nodes(s->d, par, node_chunk(s), s->stream, early), "node update");
+        if (objects) LBIB_CUDA(s, launch_nodes(s->d, par, s->node_threads, s->stream, early), "node update");
         if (objects && s->overlap) {
             LBIB_CUDA(s, cudaEventRecord(s->ev_nodes, s->stream), "event");
             LBIB_CUDA(s, cudaStreamWaitEvent(s->aux, s->ev_nodes, 0), "event");
@@ -1362,9 +1362,9 @@ lbib_status lbib_set_tuning(lbib_sim *s, int key, int value) {
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_MEMBRANE_THREADS) {
-        if (value < 32 || value > IB_THREADS || value % 32) return fail(s, LBIB_ERR_ARG, "membrane threads must be a multiple of 32 in [32, 256]");
+        if (value != 0 && (value < 32 || value > IB_THREADS || value % 32))
+            return fail(s, LBIB_ERR_ARG, "membrane threads must be 0 or a multiple of 32 in [32, 256]");
         s->membrane_threads = value;
-        s->membrane_auto = s->membrane_threads == 192 && s->membrane_group == 1;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_MEMBRANE_CLUSTERS) {
@@ -1380,14 +1380,12 @@ lbib_status lbib_set_tuning(lbib_sim *s, int key, int value) {
     if (key == LBIB_TUNE_MEMBRANE_GROUP) {
         if (value < 1 || value > 15) return fail(s, LBIB_ERR_ARG, "membrane group must be in [1, 15]");
         s->membrane_group = value;
-        s->membrane_auto = s->membrane_threads == 192 && s->membrane_group == 1;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_NODE_THREADS) {
         if (value != 32 && value != 64 && value != 128 && value != 256)
             return fail(s, LBIB_ERR_ARG, "node threads must be 32, 64, 128 or 256");
         s->node_threads = value;
-        s->node_auto = value == IB_THREADS_DEFAULT;
         return LBIB_OK;
     }
     if (key == LBIB_TUNE_EARLY_LAUNCH) {

@@ -42,7 +42,12 @@ namespace lbib {
 constexpr int NQ = 19;
 constexpr int FLUID_THREADS = 256;
 constexpr int IB_THREADS = 256;          // largest LBIB_TUNE_MEMBRANE_THREADS
-constexpr int IB_THREADS_DEFAULT = 256;  // node kernel block (LBIB_TUNE_NODE_THREADS)
+// Nodes per block of the node kernel (LBIB_TUNE_NODE_THREADS).  A node waits for two
+// rounds of memory, one after the other, and small blocks leave and refill an
+// SM one by one (steps with 32 / 64 / 128: 200 cells 256x128x128 FP16 82.9 / 83.1 /
+// 83.3 us, 2000 cells FP32 934 / 934 / 937, 24 serving requests 229.9 / 230.6 /
+// 231.8; 256 was slower still).
+constexpr int NODE_CHUNK_DEFAULT = 64;
 constexpr int MAX_TEMPLATE_NODES = 5120;  // 11 floats of shared memory per node
 constexpr int ACTIVE_RESET_STEPS = 128;    // period of the active-cell re-marking
 

@@ -79,12 +79,10 @@ struct lbib_sim {
     cudaStream_t side = nullptr;
     bool overlap = true;                // membrane of step t+1 on `aux` during fluid of step t
     int membrane_clusters = 0;          // clusters of the membrane kernel (0: one per object)
-    int membrane_threads = 192;         // block size of the membrane kernel (per object) ...
-    bool membrane_auto = true;          // ... unless it and the group have their defaults: membrane_threads()
+    int membrane_threads = 0;           // threads per object of the membrane kernel (0: by the rule)
     int membrane_group = 1;             // objects per block of the membrane kernel
     bool early_launch = false;          // programmatic dependent launch of the node and fluid kernels
-    int node_threads = lbib::IB_THREADS_DEFAULT;  // nodes per block of the node kernel ...
-    bool node_auto = true;                        // ... unless it has its default: node_chunk()
+    int node_threads = lbib::NODE_CHUNK_DEFAULT;  // nodes per block of the node kernel
 
     double rep_obj[3] = {0, 1, 0};      // soft-sphere repulsion (a, n, cutoff) between objects
     double rep_wall[3] = {0, 1, 0};     // and against the walls
@@ -116,10 +114,7 @@ lbib_status sim_upload(lbib_sim *s);
 lbib_status sim_prepare_step(lbib_sim *s);
 lbib_status sim_edge_scratch(lbib_sim *s);
 cudaError_t sim_remark(lbib_sim *s, cudaStream_t st);
-// Nodes per block of the node kernel: 64 while the knob has its default.  A node waits for two
-// rounds of memory, one after the other, and small blocks leave and refill an
-// SM one by one (steps with 32 / 64 / 128: 200 cells 256x128x128 FP16 82.9 / 83.1 /
-// 83.3 us, 2000 cells FP32 934 / 934 / 937, 24 serving requests 229.9 / 230.6 /
-// 231.8; 256 was slower still).
-inline int node_chunk(const lbib_sim *s) { return s->node_auto ? 64 : s->node_threads; }
+// The rule of membrane_threads() holds for one object per block; 192 threads where it does not.
+inline bool membrane_by_rule(const lbib_sim *s) { return s->membrane_threads == 0 && s->membrane_group == 1; }
+inline int membrane_block(const lbib_sim *s) { return s->membrane_threads ? s->membrane_threads : 192; }
 }  // namespace lbib

@@ -18,7 +18,8 @@ floating-point atomics, only the speed:
 candidate and keeps the fastest, one knob group at a time (membrane
 clusters and overlap, then threads per object together with objects per
 membrane block, then the node chunk, then the fluid kernel, then early
-launch, each group searched with the best choice of the groups before it).  Results are cached by a key of
+launch, each group searched with the best choice of the groups before it, which
+stays where nothing in the group was faster).  Results are cached by a key of
 the workload's shape (number of simulations, box-size class, node-count
 class, storage precisions, batched or not), so simulations of the same class
 reuse the choice.  Tuning advances the simulations it times; callers tune on
@@ -36,7 +37,8 @@ KNOBS = (("cluster", lbib.LBIB_TUNE_IB_CLUSTER), ("overlap", lbib.LBIB_TUNE_OVER
          ("membrane_threads", lbib.LBIB_TUNE_MEMBRANE_THREADS), ("membrane_group", lbib.LBIB_TUNE_MEMBRANE_GROUP),
          ("node_threads", lbib.LBIB_TUNE_NODE_THREADS), ("fluid_kernel", lbib.LBIB_TUNE_FLUID_KERNEL),
          ("early_launch", lbib.LBIB_TUNE_EARLY_LAUNCH))
-DEFAULT = {"cluster": 1, "overlap": 1, "membrane_threads": 192, "membrane_group": 1, "node_threads": 256,
+# membrane_threads 0: the library's rule, which also takes blocks larger than the knob's
+DEFAULT = {"cluster": 1, "overlap": 1, "membrane_threads": 0, "membrane_group": 1, "node_threads": 64,
            "fluid_kernel": 0, "early_launch": 0}
 
 
@@ -108,7 +110,7 @@ def autotune(sims, steps=32, batched=None, **search):
     if key in _CACHE:
         apply(sims, _CACHE[key][0])
         return _CACHE[key]
-    best = dict(DEFAULT)
+    best, t_best = dict(DEFAULT), float("inf")
     timing = {}
     for names, values in candidates(sims, batched, **search):
         group_t = {}
@@ -118,7 +120,10 @@ def autotune(sims, steps=32, batched=None, **search):
             t = _time(sims, steps, batched)
             group_t[vals] = t
             timing[",".join(f"{n}={v}" for n, v in zip(names, vals))] = t
-        best.update(dict(zip(names, min(group_t, key=group_t.get))))
+        vals = min(group_t, key=group_t.get)
+        if group_t[vals] < t_best:
+            best.update(zip(names, vals))
+            t_best = group_t[vals]
     apply(sims, best)
     _CACHE[key] = (best, timing)
     return _CACHE[key]
