@@ -220,9 +220,12 @@ lbib_status sim_upload(lbib_sim *s) {
             s->fext_dirty = true;
         }
         std::vector<MemDev> mem(nobj);
+        s->scal_bytes = 0;
         for (int o = 0; o < nobj; ++o) {
             mem[o] = s->tpl_mem_dev[s->objs[o].tid];
             mem[o].first = s->objs[o].first;
+            mem[o].scal = (unsigned)(s->scal_bytes / 16);
+            s->scal_bytes += membrane_scalar_bytes(mem[o].ne);
         }
         if (nobj > 0)
             LBIB_CUDA(s, cudaMemcpyAsync(s->d_mem, mem.data(), nobj * sizeof(MemDev), cudaMemcpyHostToDevice, s->stream),
@@ -354,7 +357,7 @@ lbib_status sim_upload(lbib_sim *s) {
 // Global memory for the edge scalars of every object, for launches that do
 // not keep them in shared memory (membrane_in_global).
 lbib_status sim_edge_scratch(lbib_sim *s) {
-    const size_t stride = align_up(membrane_scalar_bytes(s->max_edges), 16), bytes = s->objs.size() * stride;
+    const size_t bytes = s->scal_bytes;
     if (bytes > s->edge_bytes) {
         if (s->d.edge_scal) cudaFree(s->d.edge_scal);
         s->d.edge_scal = nullptr;
@@ -362,7 +365,6 @@ lbib_status sim_edge_scratch(lbib_sim *s) {
         LBIB_CUDA(s, cudaMalloc(&s->d.edge_scal, bytes), "edge scalars");
         s->edge_bytes = bytes;
     }
-    s->d.edge_stride = stride;
     return LBIB_OK;
 }
 
@@ -421,9 +423,11 @@ int64_t lbib_footprint_bytes(const lbib_fluid_params *p, int64_t n_nodes, int64_
     if (!p) return -1;
     FluidLayout L;
     if (!fluid_layout(*p, L)) return -1;
-    // nodes: X, V (hi + lo FP32), membrane force, owner; templates: triangle,
-    // edge and bending records
-    return (int64_t)L.total + n_nodes * 64 + n_tri_total * (16 + 3 * 16 + 4 * 20);
+    // nodes: X, V (hi + lo FP32), membrane force, owner, and the scalars of 3 edges
+    // and 2 triangles a node, which launches of large or shared objects keep in
+    // memory (closed meshes without handles have no more); templates: triangle,
+    // edge and walk records
+    return (int64_t)L.total + n_nodes * (64 + 3 * 8 + 2 * 4) + n_tri_total * (16 + 3 * 16 + 4 * 20);
 }
 
 lbib_status lbib_create(const lbib_fluid_params *p, void *stream, lbib_sim **out) {

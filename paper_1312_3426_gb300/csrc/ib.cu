@@ -41,7 +41,7 @@ bool membrane_in_global(int max_nodes, int max_edges, int cluster) {
     return cluster > 1 || ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX;
 }
 
-size_t membrane_scalar_bytes(int max_edges) { return ib_scalar_bytes(max_edges); }
+size_t membrane_scalar_bytes(int edges) { return (ib_scalar_bytes(edges) + 15) & ~(size_t)15; }
 
 // The membrane kernel takes about 10 us plus 3.5 us for every round of the
 // block over the edges (beside the fluid kernel; a level-3 cell of 1920

@@ -115,7 +115,9 @@ struct alignas(16) MemDev {
     int edge_stride, flags;  // MEM_ALTITUDE: local-area force along the altitudes (else centroid -> vertex)
     float ks, kb, kal, kag;
     double Sg0, V0;
-    float kv, pad[3];
+    float kv;
+    unsigned scal;  // the object's place in SimDev::edge_scal, in 16 bytes
+    float pad[2];
 };
 
 // One object: its template, first global node, node count and 1/m.
@@ -163,8 +165,7 @@ struct SimDev {
     float4 *ufield;
     float *Xh, *Xl, *Vh, *Vl; // [3][nn_total] each
     float *Fel;               // [3][nn_total] membrane force of the current step
-    char *edge_scal;          // [nobj][edge_stride] edge and triangle scalars, where shared memory does not serve
-    size_t edge_stride;       // bytes
+    char *edge_scal;          // edge and triangle scalars of every object, where shared memory does not serve
     const int *node_obj;      // [nn_total] object of each node
     int nn_total, nobj;
     const ObjDev *obj;
@@ -313,7 +314,7 @@ cudaError_t launch_membrane(const SimDev &s, int max_nodes, int max_edges, int c
 // SimDev::edge_scal: several blocks per object, or more than one block's
 // shared memory holds
 bool membrane_in_global(int max_nodes, int max_edges, int cluster);
-size_t membrane_scalar_bytes(int max_edges);  // per object
+size_t membrane_scalar_bytes(int edges);  // of an object, a multiple of 16
 // Threads per object of a membrane launch of nobj objects (one per block)
 // beside a fluid update of fluid_us microseconds (0: nothing beside it).
 int membrane_threads(int nobj, int max_edges, double fluid_us);

@@ -30,7 +30,8 @@ struct lbib_sim {
     size_t tpl_bytes = 0;
     int max_nodes = 0;                  // of the largest object (templates may have none)
     int max_edges = 0;
-    size_t edge_bytes = 0;              // of SimDev::edge_scal
+    size_t scal_bytes = 0;              // what SimDev::edge_scal takes for the objects
+    size_t edge_bytes = 0;              // ... and what it has (0 until a launch needs it)
 
     std::vector<lbib::ObjDev> objs;
     int nn_total = 0;
