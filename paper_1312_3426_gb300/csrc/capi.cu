@@ -10,6 +10,7 @@
 #include <cstdio>
 #include <cstring>
 #include <initializer_list>
+#include <mutex>
 #include <string>
 #include <vector>
 
@@ -104,6 +105,32 @@ void rotation_zyx(const double r[3], double R[3][3]) {
     R[2][0] = -sy;
     R[2][1] = cy * sx;
     R[2][2] = cy * cx;
+}
+
+// The live simulations of the process, so that one knows whether others may run beside it.
+std::mutex live_mu;
+lbib_sim *live = nullptr;
+
+void live_enter(lbib_sim *s) {
+    std::lock_guard<std::mutex> lock(live_mu);
+    s->live_next = live;
+    if (live) live->live_prev = s;
+    live = s;
+}
+
+void live_leave(lbib_sim *s) {
+    std::lock_guard<std::mutex> lock(live_mu);
+    (s->live_prev ? s->live_prev->live_next : live) = s->live_next;
+    if (s->live_next) s->live_next->live_prev = s->live_prev;
+}
+
+// Whether another simulation on the device has another stream.
+bool streams_beside(const lbib_sim *s) {
+    const auto handle = [](const lbib_sim *x) { return x->stream == cudaStreamLegacy ? nullptr : x->stream; };
+    std::lock_guard<std::mutex> lock(live_mu);
+    for (const lbib_sim *x = live; x; x = x->live_next)
+        if (x->device == s->device && handle(x) != handle(s)) return true;
+    return false;
 }
 
 }  // namespace
@@ -507,12 +534,14 @@ lbib_status lbib_create(const lbib_fluid_params *p, void *stream, lbib_sim **out
         delete s;
         return LBIB_ERR_CUDA;
     }
+    live_enter(s);
     *out = s;
     return LBIB_OK;
 }
 
 void lbib_destroy(lbib_sim *s) {
     if (!s) return;
+    live_leave(s);
     cudaSetDevice(s->device);
     cudaStreamSynchronize(s->stream);
     if (s->aux) {
@@ -929,7 +958,8 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
 // whose launch knobs have their defaults, while no step is sampled.
 static bool many_steps(const lbib_sim *s) {
     return s->overlap && membrane_by_rule(s) && s->cluster == 1 && s->membrane_clusters == 0 && !s->early_launch &&
-           s->node_threads == NODE_CHUNK_DEFAULT && !s->prof_on && !s->many_refused && s->d.fkern != 2 && steps_fit(s->d, s->max_nodes, s->max_edges);
+           s->node_threads == NODE_CHUNK_DEFAULT && !s->prof_on && !s->many_refused && s->d.fkern != 2 &&
+           steps_fit(s->d, s->max_nodes, s->max_edges, streams_beside(s));
 }
 
 lbib_status lbib_step(lbib_sim *s, int n) {

@@ -298,7 +298,8 @@ cudaError_t launch_mass_partials(const SimDev &s, int pop_par, double *part, int
 // n steps from step t on in one cooperative launch, where steps_fit; sync:
 // 192 device bytes of counters.  The membrane forces of the first step's
 // positions are in Fel, and those of the final positions will be.
-bool steps_fit(const SimDev &s, int max_nodes, int max_edges);
+// shared: simulations on other streams may run beside it
+bool steps_fit(const SimDev &s, int max_nodes, int max_edges, bool shared);
 cudaError_t launch_steps(const SimDev &s, int max_nodes, int max_edges, long long t, int n, unsigned *sync,
                          cudaStream_t st);
 

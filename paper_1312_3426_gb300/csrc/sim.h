@@ -16,6 +16,7 @@ struct lbib_sim {
     uint64_t serial = 0;         // unique per simulation of the process (an address may be reused)
     cudaStream_t stream = nullptr;
     int device = 0;
+    lbib_sim *live_next = nullptr, *live_prev = nullptr;  // the live simulations of the process
     std::string err;
     lbib_status sticky = LBIB_OK;
 

@@ -161,8 +161,19 @@ static int steps_fluid_blocks(const SimDev &s, int max_edges) {
 //   10 bodies with repulsion among posts FP16: 199x50x30 12.8 / 32.4, 200x64x64 26.0 / 33.8
 // beyond (6.4 rounds at 96x96x96 FP32 30.6 / 28.8, 9.5 at 160x128x96 FP16 37.3 /
 // 37.4) they are equal or worse.
-bool steps_fit(const SimDev &s, int max_nodes, int max_edges) {
+//
+// Beside simulations on other streams, half of the SMs at most, so that two such
+// launches fit: the blocks hold their SMs while they wait, where separate launches
+// fill one simulation's gaps with another's work.  us a simulation and step on 8
+// streams, one launch against separate ones:
+//   sphere 40x20x20                 2.1 /  4.1    3 cells 64x48x48 FP16  4.3 /  4.8
+// and with more SMs
+//   20 cells 117x70x66 FP32        17.0 / 15.0    128x64x64 FP16  12.9 / 11.2
+//   20 cells 160x96x96 FP16        29.1 / 22.8    8 level-4 cells 128x64x64 FP32 28.1 / 15.5
+//   no objects 64x48x48             5.2 /  2.9    101x37x53  5.7 / 4.4    128x96x96 FP16 16.7 / 15.5
+bool steps_fit(const SimDev &s, int max_nodes, int max_edges, bool shared) {
     const int sms = device_sms();
+    if (shared && 2 * (s.nobj + steps_fluid_blocks(s, max_edges)) > sms) return false;
     if ((s.rep_on && s.nobj > REPEL_MAX_OBJECTS) || (s.nobj > 0 && ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX)) return false;
     const int tiles = steps_tiles(s, max_edges);
     if (s.nobj == 0) return tiles >= 32 && tiles <= 5 * sms;
