@@ -297,13 +297,15 @@ LBIB_API lbib_status lbib_profile_enable(lbib_sim *sim, int on);
 LBIB_API lbib_status lbib_profile_read(lbib_sim *sim, double out[6]);
 
 /* Check of the device-side bounded waits (the warp-specialised fluid
- * kernel's pipeline waits give up after about 2 s, set the status the next
+ * kernel's pipeline waits give up after about 2 s, the barriers of a launch of
+ * many steps after 10 s of waiting; they set the status the next
  * call reports as LBIB_ERR_TIMEOUT, and leave the context usable instead
- * of hanging).  Runs one such wait on the current device, on a barrier that
+ * of hanging).  Runs one wait of each kind on the current device, on a barrier that
  * nothing completes (arrive = 0) or that its own thread completes first
- * (arrive = 1), bounded by `seconds`; *timed_out = 1 when the wait gave up.
- * Returns after the wait.  LBIB_ERR_ARG for a null output or seconds outside
- * (0, 10]; LBIB_ERR_CUDA when the device calls fail. */
+ * (arrive = 1), bounded by `seconds` each; *timed_out = 1 when the waits gave up.
+ * Returns after the waits.  LBIB_ERR_ARG for a null output or seconds outside
+ * (0, 10]; LBIB_ERR_CUDA when the device calls fail; LBIB_ERR_TIMEOUT when one wait
+ * gave up and the other did not. */
 LBIB_API lbib_status lbib_check_bounded_wait(double seconds, int arrive, int *timed_out);
 
 /* Total fluid mass sum_cells sum_i f_i, an FP64 reduction on the GPU. */

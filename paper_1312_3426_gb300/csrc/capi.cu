@@ -1241,18 +1241,21 @@ lbib_status lbib_fluid_mass(lbib_sim *s, double *mass) {
 // a stack array.
 lbib_status lbib_check_bounded_wait(double seconds, int arrive, int *timed_out) {
     if (!timed_out || !(seconds > 0.0) || seconds > 10.0) return LBIB_ERR_ARG;
-    uint32_t *d = nullptr, h = 0;
+    uint32_t *d = nullptr, h[2] = {0, 0};  // a status word for each wait, the counter of the second
     cudaStream_t st = nullptr;
+    const unsigned long long ns = (unsigned long long)(seconds * 1e9);
     cudaError_t e = cudaStreamCreateWithFlags(&st, cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMalloc(&d, sizeof(uint32_t));
-    if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, sizeof(uint32_t), st);
-    if (e == cudaSuccess) e = run_wait_probe(d, (unsigned long long)(seconds * 1e9), arrive ? 1 : 0, st);
-    if (e == cudaSuccess) e = cudaMemcpyAsync(&h, d, sizeof(uint32_t), cudaMemcpyDeviceToHost, st);
+    if (e == cudaSuccess) e = cudaMalloc(&d, 3 * sizeof(uint32_t));
+    if (e == cudaSuccess) e = cudaMemsetAsync(d, 0, 3 * sizeof(uint32_t), st);
+    if (e == cudaSuccess) e = run_wait_probe(d, ns, arrive ? 1 : 0, st);
+    if (e == cudaSuccess) e = run_steps_wait_probe(d + 1, d + 2, ns, arrive ? 1 : 0, st);
+    if (e == cudaSuccess) e = cudaMemcpyAsync(h, d, sizeof(h), cudaMemcpyDeviceToHost, st);
     if (e == cudaSuccess) e = cudaStreamSynchronize(st);
     if (d) cudaFree(d);
     if (st) cudaStreamDestroy(st);
     if (e != cudaSuccess) return LBIB_ERR_CUDA;
-    *timed_out = (h & ST_TIMEOUT) ? 1 : 0;
+    if ((h[0] ^ h[1]) & ST_TIMEOUT) return LBIB_ERR_TIMEOUT;
+    *timed_out = (h[0] & ST_TIMEOUT) ? 1 : 0;
     return LBIB_OK;
 }
 

@@ -302,6 +302,8 @@ cudaError_t launch_mass_partials(const SimDev &s, int pop_par, double *part, int
 bool steps_fit(const SimDev &s, int max_nodes, int max_edges, bool shared);
 cudaError_t launch_steps(const SimDev &s, int max_nodes, int max_edges, long long t, int n, unsigned *sync,
                          cudaStream_t st);
+// the bounded-wait check of its barriers (c: a zero counter)
+cudaError_t run_steps_wait_probe(uint32_t *status, unsigned *c, unsigned long long bound_ns, int arrive, cudaStream_t st);
 
 // ---- launchers (ib.cu) -----------------------------------------------------
 // membrane part: clusters of `cluster` blocks, one per object or at most

@@ -19,11 +19,12 @@
 // launch), added to after a block barrier and a fence, read with acquire by
 // one thread before a block barrier.  All blocks are resident (cooperative
 // launch) and arrive at every barrier in order, so every wait ends; as
-// everywhere it is bounded by the global timer all the same: one that runs out
+// everywhere it is bounded all the same (bounded_wait.h): one that runs out
 // sets ST_TIMEOUT and the block leaves.  What another block writes during the
 // launch is read through the L2 (populations, velocity samples, mask, forces,
 // and the positions of an object by its membrane block); a node's own state
 // stays with its warp.
+#include "bounded_wait.h"
 #include "fluid_core.cuh"
 #include "ib_core.cuh"
 
@@ -44,18 +45,23 @@ __device__ __forceinline__ unsigned ld_acquire(const unsigned *p) {
     return v;
 }
 
+__device__ __forceinline__ unsigned long long steps_clock() {
+    unsigned long long t;
+    asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+    return t;
+}
+
 // Until *c has reached target (all threads of the block call it); false when
 // the bound ran out.
-__device__ __forceinline__ bool steps_wait(const SimDev &s, const unsigned *c, unsigned target) {
+__device__ __forceinline__ bool steps_wait(uint32_t *status, const unsigned *c, unsigned target,
+                                           unsigned long long bound_ns = STEPS_WAIT_NS) {
     bool late = false;
     if (threadIdx.x == 0 && ld_acquire(c) < target) {
-        unsigned long long t0, t1;
-        asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t0));
+        WaitClock clock;
+        clock.start(steps_clock());
         for (unsigned i = 1; ld_acquire(c) < target; ++i) {
-            if ((i & 1023u) != 0u) continue;
-            asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t1));
-            if (t1 - t0 > STEPS_WAIT_NS) {
-                atomicOr(s.status, ST_TIMEOUT);
+            if ((i & 1023u) == 0u && clock.over(steps_clock(), bound_ns)) {
+                atomicOr(status, ST_TIMEOUT);
                 late = true;
                 break;
             }
@@ -72,6 +78,18 @@ __device__ __forceinline__ void steps_signal(unsigned *c) {
     }
 }
 
+// Check of the wait itself: one block waits for a counter that nothing adds to, or
+// that it has added to first.
+__global__ void k_steps_wait_probe(uint32_t *status, unsigned *c, unsigned long long bound_ns, int arrive) {
+    if (arrive) steps_signal(c);
+    steps_wait(status, c, 1u, bound_ns);
+}
+
+cudaError_t run_steps_wait_probe(uint32_t *status, unsigned *c, unsigned long long bound_ns, int arrive, cudaStream_t st) {
+    k_steps_wait_probe<<<1, 64, 0, st>>>(status, c, bound_ns, arrive);
+    return cudaGetLastError();
+}
+
 // PAIR: two cells per thread (BC: nx odd), else one (BC: obstacles or an inlet)
 template <typename T, bool PAIR, bool BC>
 __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, long long t0, int n, unsigned *sync) {
@@ -83,19 +101,19 @@ __global__ void __launch_bounds__(STEPS_THREADS<T, PAIR>, 1) k_steps(SimDev s, l
     for (int k = 0; k < n; ++k) {
         const long long t = t0 + k;
         const int par = (int)(t & 1);
-        if (k > 0 && !steps_wait(s, done, blocks * (unsigned)k)) return;
+        if (k > 0 && !steps_wait(s.status, done, blocks * (unsigned)k)) return;
         if (nobj > 0) {
             constexpr int L = NODE_LANES<MODE_MANY>;
             for (int i = 32 / L * (int)((threadIdx.x >> 5) * blocks + blockIdx.x); i < s.nn_total; i += THREADS / L * (int)blocks)
                 node_step<MODE_MANY>(s, i + (int)(threadIdx.x & 31) / L, par);
             steps_signal(nodes_done);
-            if (!steps_wait(s, nodes_done, blocks * (unsigned)(k + 1))) return;
+            if (!steps_wait(s.status, nodes_done, blocks * (unsigned)(k + 1))) return;
         }
         if (b < nobj) {
             membrane_object<false, MODE_MANY>(s, b, steps_smem, BlockTeam());
             if (s.rep_on) {  // the other objects' boxes
                 steps_signal(boxes_done);
-                if (!steps_wait(s, boxes_done, (unsigned)nobj * (unsigned)(k + 1))) return;
+                if (!steps_wait(s.status, boxes_done, (unsigned)nobj * (unsigned)(k + 1))) return;
                 repel_object(s, b, steps_smem);
             }
         } else {
