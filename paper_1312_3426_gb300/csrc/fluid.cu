@@ -108,8 +108,11 @@ static cudaError_t launch_fluid_t(const SimDev &s, int par, uint32_t seed, int b
         if (pdl) return launch_dep(k_fluid<T, true, true>, b, FLUID_THREADS, st, true, d, seed, pf);
         return launch_dep(k_fluid<T, true, false>, b, FLUID_THREADS, st, false, d, seed, pf);
     }
-    if (pdl) return launch_dep(k_fluid<T, false, true>, b, FLUID_THREADS, st, true, d, seed, pf);
-    return launch_dep(k_fluid<T, false, false>, b, FLUID_THREADS, st, false, d, seed, pf);
+    if constexpr (sizeof(T) == 2) {
+        if (pdl) return launch_dep(k_fluid<T, false, true>, b, FLUID_THREADS, st, true, d, seed, pf);
+        return launch_dep(k_fluid<T, false, false>, b, FLUID_THREADS, st, false, d, seed, pf);
+    }
+    return cudaErrorInvalidValue;  // FP32 without obstacles or an inlet takes two cells per thread
 }
 
 cudaError_t launch_fluid(const SimDev &s, int par, long long t, cudaStream_t st, bool pdl) {
