@@ -167,10 +167,14 @@ static int steps_fluid_blocks(const SimDev &s, int max_edges) {
 }
 
 // Up to 8 rounds of the fluid blocks (6 of the FP32 two-cells blocks, which
-// have 16 warps; without objects 32 tiles to 5 rounds), and objects on half of
-// the SMs at most.  us a step, one launch against separate ones:
+// have 16 warps; without objects 5), and objects on half of the SMs at most.
+// Without objects from 32 tiles on, and from 64 where a thread has two cells of one
+// row (16 bits, even width): a separate launch takes 4.1 us, or 6.2 where the
+// kernel is longer, a step of a launch 4.0 to 4.7.  us a step, one launch against separate ones:
 //   sphere 40x20x20                 8.2 / 12.7
 //   no objects 101x37x53            5.7 /  6.2    128x96x96 FP16  16.7 / 18.6
+//     30x32x31 FP32                 4.0 /  4.1    FP16 4.6 / 4.1; 40x40x40 4.0 / 5.7, 4.7 / 4.1; 41x40x39 FP16 5.3 / 6.2
+//     48x40x40 FP16                 4.7 /  4.1    48x48x48 4.9 / 5.1, 64x48x48 4.8 / 6.2
 //   3 cells 64x48x48 FP16          11.5 / 20.5
 //   20 cells 117x70x66 FP32        17.0 / 22.5
 //   20 cells 128x64x64 FP32        16.0 / 22.8    FP16  12.9 / 22.1
@@ -194,7 +198,10 @@ bool steps_fit(const SimDev &s, int max_nodes, int max_edges, bool shared) {
     if (shared && 2 * (s.nobj + steps_fluid_blocks(s, max_edges)) > sms) return false;
     if ((s.rep_on && s.nobj > REPEL_MAX_OBJECTS) || (s.nobj > 0 && ib_smem_bytes(max_nodes, max_edges) > IB_SMEM_MAX)) return false;
     const int tiles = steps_tiles(s, max_edges);
-    if (s.nobj == 0) return tiles >= 32 && tiles <= 5 * sms;
+    if (s.nobj == 0) {
+        const bool row = s.prec != LBIB_POP_F32 && steps_pair(s, max_edges) && s.nx % 2 == 0;
+        return tiles >= (row ? 64 : 32) && tiles <= 5 * sms;
+    }
     const int rounds = s.prec == LBIB_POP_F32 && steps_pair(s, max_edges) ? 6 : 8;
     return 2 * s.nobj <= sms && tiles <= rounds * (sms - s.nobj);
 }

@@ -62,6 +62,16 @@ def test_one_launch_leaves_room_for_other_streams(one_launch):
     same.close()
 
 
+@pytest.mark.parametrize("box,prec,one", [((48, 40, 40), "f16s", False), ((48, 48, 48), "f16s", True),
+                                          ((41, 40, 39), "bf16s", True), ((40, 40, 40), "f32", True)])
+def test_small_channels_without_objects(one_launch, box, prec, one):
+    """Where a launch of many steps starts to be faster (figures at steps_fit)."""
+    g = lbib.Sim(*box, body_force=(1e-5, 0, 0), precision=prec, pop_scale_log2=0 if prec == "f32" else 12)
+    g.fluid_init()
+    assert one_launch(g) == one
+    g.close()
+
+
 def test_simulations_at_once_equal_alone():
     scs = [scenes.channel_sphere(), scenes.Scene("free", 64, 64, 64, body_force=(2e-5, 0.0, 1e-5)),
            scenes.channel_sphere(), scenes.Scene("odd", 41, 30, 37, body_force=(1e-5, 0.0, 2e-5))]
