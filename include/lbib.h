@@ -424,7 +424,8 @@ LBIB_API lbib_status lbib_server_stats(const lbib_server *srv, int64_t out[4]);
  * that kernel does not write, and waits for it before the rest), 0 (default)
  * launches them one after the other; lbib_batch_step ignores it.
  * With every knob at its default, a small simulation (see csrc/steps.cu) runs
- * the steps of one lbib_step call in one launch.
+ * the steps of one lbib_step call in one launch (while simulations on other streams
+ * exist, one that needs half of the SMs at most).
  * Results do not depend on the knobs beyond the order of
  * floating-point atomics (the three 16-bit kernels give identical
  * populations).  LBIB_ERR_ARG for an unknown key or an out-of-range value. */

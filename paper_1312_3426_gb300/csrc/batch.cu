@@ -2,12 +2,13 @@
 //
 // A step of the batch is the step of lbib_step (see capi.cu) with every
 // kernel launched once for all simulations over a flat work list:
-//   node kernel      one block per (simulation, run of IB_THREADS nodes)
-//   fluid kernel     one block per (simulation, run of FLUID_THREADS cells),
-//                    one launch per storage type present
-//   membrane kernel  one thread-block cluster per (simulation, object), on a
-//                    second stream while the fluid kernel runs (it prepares
-//                    the next step)
+//   node kernel      one block per (simulation, run of nodes of the chunk knob)
+//   fluid kernel     one block per (simulation, run of FLUID_THREADS cells or
+//                    PAIR_THREADS pairs), one launch per variant present (fluid_group)
+//   membrane kernel  one block (or cluster, or group of a block's threads) per
+//                    (simulation, object), in one or two launches by size on
+//                    streams of their own while the fluid kernel runs (it
+//                    prepares the next step)
 // so the launch count per step does not grow with the number of
 // simulations, and small simulations fill the GPU together.  Every block
 // reads its simulation's descriptor and step counter from device arrays;
@@ -20,7 +21,8 @@
 // The per-item device code is the code of the single-simulation kernels, so
 // a simulation advanced in a batch computes what lbib_step computes for it
 // alone, up to the order of the FP32 atomics of the spreading and of the
-// membrane-force sums (as between two runs of lbib_step).
+// repulsion (as between two runs of lbib_step); membrane forces are sums of a
+// fixed order.
 #include <cuda_runtime.h>
 
 #include <algorithm>
@@ -63,7 +65,7 @@ __global__ void __launch_bounds__(FLUID_THREADS, 5)
     fluid_block<T, BC, MODE_PLAIN>(s, (int)(t & 1), it.y * FLUID_THREADS, step_seed(t));
 }
 
-// Plain boundaries, 16-bit storage: two cells per thread (ODD: nx odd).
+// 16-bit storage without obstacles or an inlet: two cells per thread (ODD: nx odd).
 template <typename T, bool ODD>
 __global__ void __launch_bounds__(PAIR_THREADS, pair_blocks<T>())
     k_batch_fluid_pair(const SimDev *__restrict__ sims, const long long *__restrict__ t_base, int step_off,
@@ -118,7 +120,7 @@ __global__ void k_batch_advance(long long *t_base, int n, int steps) {
 struct BatchPlan {
     std::vector<lbib_sim *> sims;
     std::vector<uint64_t> serial;  // identity of each simulation (addresses can be reused)
-    std::vector<int> nobj, nn, group;  // group: fluid kernel variant (2 * precision + BC)
+    std::vector<int> nobj, nn, group;  // group: fluid kernel variant (fluid_group)
     std::vector<SimDev> dev;  // descriptors the device copy holds
     int cluster = 0, device = -1, mthreads = IB_THREADS, nthreads = NODE_CHUNK_DEFAULT, mgroup = 1;
     SimDev *d_sims = nullptr;

@@ -946,6 +946,15 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
     return LBIB_OK;
 }
 
+// Whether lbib_step runs its steps in one launch (steps.cu): a small simulation
+// whose launch knobs have their defaults, while no step is sampled (beside
+// simulations on other streams, one that needs half of the SMs at most).
+static bool many_steps(const lbib_sim *s) {
+    return s->overlap && membrane_by_rule(s) && s->cluster == 1 && s->membrane_clusters == 0 && !s->early_launch &&
+           s->node_threads == NODE_CHUNK_DEFAULT && !s->prof_on && !s->many_refused && s->d.fkern != 2 &&
+           steps_fit(s->d, s->max_nodes, s->max_edges, streams_beside(s));
+}
+
 // One step is: coupling part of the object update (node kernel), then the
 // fluid step; the membrane part of the NEXT step depends only on the node
 // positions the node kernel wrote, so (overlap on) it runs on the second
@@ -954,14 +963,6 @@ static lbib_status launch_membrane_timed(lbib_sim *s, cudaStream_t st) {
 //   aux:    wait ev_nodes, membrane(t+1) -> ev_membrane
 // and `stream` has caught up with `aux` when the call returns.  With overlap
 // off every step is membrane(t), nodes(t), fluid(t) on `stream`.
-// Whether lbib_step runs its steps in one launch (steps.cu): a small simulation
-// whose launch knobs have their defaults, while no step is sampled.
-static bool many_steps(const lbib_sim *s) {
-    return s->overlap && membrane_by_rule(s) && s->cluster == 1 && s->membrane_clusters == 0 && !s->early_launch &&
-           s->node_threads == NODE_CHUNK_DEFAULT && !s->prof_on && !s->many_refused && s->d.fkern != 2 &&
-           steps_fit(s->d, s->max_nodes, s->max_edges, streams_beside(s));
-}
-
 lbib_status lbib_step(lbib_sim *s, int n) {
     LBIB_GUARD(s);
     if (n < 0) return fail(s, LBIB_ERR_ARG, "negative step count");

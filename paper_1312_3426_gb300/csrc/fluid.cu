@@ -1,8 +1,8 @@
 // Fluid kernels: fused pull-stream + collide (Eq. lbequation), read-outs,
 // checkpoint conversion and the FP64 mass reduction.
 //
-// One thread updates one fluid cell, or two x-adjacent ones where nx is even
-// and there are no obstacles and no inlet.  For each of the 19 directions it pulls
+// One thread updates two consecutive fluid cells, or one where there are
+// obstacles or an inlet.  For each of the 19 directions it pulls
 // the post-collision value of the previous step from the neighbour the
 // population comes from (periodic in x and z, and in y without walls); a
 // population that would come from a solid row is the cell's own opposite
@@ -16,7 +16,7 @@
 //
 // Memory traffic per fluid cell: 19 loads + 19 stores of the storage type
 // (152 B in FP32, 76 B in FP16/BF16), plus one 4-byte mask word per 32
-// cells for each of the three masks, plus 16 B reads/writes only at cells
+// cells (beside obstacles two more), plus 16 B reads/writes only at cells
 // touched by the immersed objects.
 #include <mutex>
 #include <type_traits>

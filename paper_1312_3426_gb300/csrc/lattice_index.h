@@ -8,6 +8,10 @@
 // rows: ny - 2 with walls, ny without).  Fluid cell index
 // f = x + nx (y' + nyf z) with y' = y - 1 with walls, y' = y without.
 //
+// The library marks, gathers and spreads through corner_cells and
+// corner_cells_side; fluid_index, halo_cell and for_each_halo (the 4x4x4 cells
+// around a corner) serve the host bounds test alone.
+//
 // Bounds, for every float input:
 //   lattice_coord   i0 in [-2^30 - 1, 2^30 + 1], so i0 + d for the small
 //                   offsets d used below never overflows

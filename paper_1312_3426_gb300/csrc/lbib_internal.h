@@ -48,7 +48,7 @@ constexpr int IB_THREADS = 256;          // largest LBIB_TUNE_MEMBRANE_THREADS
 // 83.3 us, 2000 cells FP32 934 / 934 / 937, 24 serving requests 229.9 / 230.6 /
 // 231.8; 256 was slower still).
 constexpr int NODE_CHUNK_DEFAULT = 64;
-constexpr int MAX_TEMPLATE_NODES = 5120;  // 11 floats of shared memory per node
+constexpr int MAX_TEMPLATE_NODES = 5120;  // k_rep_forces: 36 bytes of shared memory a node
 constexpr int ACTIVE_RESET_STEPS = 128;    // period of the active-cell re-marking
 
 // D3Q19 directions of this library: rest, the 6 axis directions in +/- pairs,
@@ -308,7 +308,7 @@ cudaError_t run_steps_wait_probe(uint32_t *status, unsigned *c, unsigned long lo
 // ---- launchers (ib.cu) -----------------------------------------------------
 // membrane part: clusters of `cluster` blocks, one per object or at most
 // max_clusters (> 0) looping over the objects (max_nodes and max_edges size
-// shared memory); coupling part: one thread per node
+// shared memory)
 // threads: block size (a multiple of 32, at most 1024)
 // group > 1: `group` objects per block of group * threads threads instead
 cudaError_t launch_membrane(const SimDev &s, int max_nodes, int max_edges, int cluster, int max_clusters, int threads,
